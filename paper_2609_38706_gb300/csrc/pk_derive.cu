@@ -80,8 +80,13 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
                 int64_t *key_off, int32_t *status) {
     __shared__ long long warp_sums[kScanThreads / 32];
     __shared__ long long tile_total;
-    pk::pdl_launch_dependents();
     pk::pdl_wait(tok_off, desc_idx, key_off, status);
+    // The chunk digests are released only here, when every earlier kernel of the stream is done: released at the
+    // start, their CTAs came up beside the previous batch's last kernels and stacked on the SMs those left free,
+    // two and more on one SM with others empty, where a small batch needs a lone warp per sub-partition.  Batches
+    // enqueued back to back, per step: 900 ragged prompts 435 -> 188 us, multi-adapter 94.5 -> 71.9 us, long
+    // context 1056 -> 947 us.
+    pk::pdl_launch_dependents();
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) key_off[0] = 0;
     bool bad = false;
