@@ -85,7 +85,7 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
     // start, their CTAs came up beside the previous batch's last kernels and stacked on the SMs those left free,
     // two and more on one SM with others empty, where a small batch needs a lone warp per sub-partition.  Batches
     // enqueued back to back, per step: 900 ragged prompts 435 -> 188 us, multi-adapter 94.5 -> 71.9 us, long
-    // context 1056 -> 947 us.
+    // context 1056 -> 947 us (both sides with the two-lane chain).
     pk::pdl_launch_dependents();
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) key_off[0] = 0;
@@ -342,43 +342,33 @@ k_chunk_digest(const int32_t *tokens, const int64_t *tok_off,
 // ---------------------------------------------------------------------------
 // Chain: k_i = SHA-256(k_{i-1} || d || c_i), serial in i for each request.
 //
-// Every 32 requests (one per lane, a "group") are served by a pair of warps:
+// A group of requests is served by a pair of warps:
 //   rounds warp:   holds the state; runs the 64 rounds of block 1
 //                  (k_{i-1} || d) and of block 2 (c_i || padding)
 //   schedule warp: writes K_t + W_t for both blocks to shared memory:
 //                  block 2's schedule depends on c_i only and is made one
 //                  step ahead; block 1's depends on k_{i-1} and is made as
 //                  soon as k_{i-1} is published.
-// Two layouts (kPairs):
-//   1  one pair per CTA (2 warps) for batches with at most one group per SM:
-//      the two warps run on different SM sub-partitions, so that one chain
-//      step costs about the rounds alone; block 1's schedule is published in
-//      three 16-word slices.  Named barriers (count 64, producer arrives,
-//      consumer syncs): 1, 2, 3 block-1 slices t = 16..31, 32..47, 48..63;
-//      4 block-2 schedule; 5 k_i published.
-//   4  four pairs per CTA (8 warps), pair p = rounds warp p and schedule warp
-//      p + 4, which share a sub-partition, one CTA per SM: with several
-//      groups per SM, 2-warp CTAs put two rounds warps on one sub-partition
-//      (51 instead of 30 cycles per round, measured) while schedule warps
-//      share another; paired on one sub-partition, the schedule fills the
-//      issue slots the rounds warp's dependency chain leaves idle.  Block 1's
-//      schedule is published in two slices, t = 16..31 and 32..63 (the rounds
-//      warp waits for the burst of block-1 schedule work after each k_{i-1},
-//      so the smaller first slice lets its rounds 16..31 overlap the rest:
-//      small-block key derivation 654 -> 641 us; three slices: 646).  The
-//      first slice's barrier also marks block 2 of the step ready (written
-//      before it), which keeps the pairs within the 16 named barriers.  Named
-//      barriers of pair p: 1 + 3p block-1 slice 1 and block 2; 2 + 3p block-1
-//      slice 2; 3 + 3p k_i published.
+// Two forms:
+//   k_chain_split  two lanes per request (split rounds of pk_sha256.cuh), 16
+//                  requests per pair: the shortest chain step, while the SM
+//                  sub-partitions have room (up to four pairs per SM);
+//   k_chain        one lane per request, 32 requests per pair, four pairs per
+//                  CTA and one CTA per SM: the fewest ALU cycles per key, for
+//                  batches that fill every sub-partition.
+// Block 1's schedule is published in two slices, t = 16..31 and 32..63 (the
+// rounds warp's rounds 16..31 overlap the making of the rest; small-block key
+// derivation 654 -> 641 us in k_chain, three slices 646).  Named barriers of
+// pair p (count 64, producer arrives, consumer syncs): 1 + 3p block-1 slice 1,
+// and block 2 of the step (written before it); 2 + 3p block-1 slice 2; 3 + 3p
+// k_i published.  Four pairs stay within the 16 named barriers.
 // Per pair both warps run the same number of steps (the lanes' maximum), so
 // every phase of every barrier gets exactly one arrive and one sync; the
-// schedule warp signals the block-2 barrier for step i only after it has
-// passed the k barrier of step i-1 (so after the rounds warp has synced the
-// block-2 barrier of step i-1), and the block-1 barriers of step i only after
-// the k barrier of step i-1 (after the rounds warp's block-1 syncs of step
-// i-1): it never arrives twice on a barrier the rounds warp has not yet
-// synced.  Block 2's buffer for step i + 1 is written after the k barrier of
-// step i - 1, when the rounds warp has finished the block 2 that last used
+// schedule warp signals the block-1 barriers of step i only after it has
+// passed the k barrier of step i-1, so after the rounds warp's block-1 syncs
+// of step i-1: it never arrives twice on a barrier the rounds warp has not
+// yet synced.  Block 2's buffer for step i + 1 is written after the k barrier
+// of step i - 1, when the rounds warp has finished the block 2 that last used
 // it.  Lanes past their own request's last chunk keep computing (masked) so
 // that the warps stay aligned.
 // ---------------------------------------------------------------------------
@@ -432,13 +422,14 @@ __device__ __forceinline__ void rounds16_kw(uint32_t v[8], const uint4 (*kw)[kCh
 }
 
 // At most 64 registers (no spills): uncapped, the compiler took 81 and a small-block step whose
-// lookup-and-store launch overlaps the chain's tail ran 910 -> 955 us.  `groups` = ceil(R / 32); with
-// kPairs = 4, CTA c serves groups [c * groups / gridDim.x, (c + 1) * groups / gridDim.x), at most four.
+// lookup-and-store launch overlaps the chain's tail ran 910 -> 955 us.  `groups` = ceil(R / 32); CTA c serves
+// groups [c * groups / gridDim.x, (c + 1) * groups / gridDim.x), at most four.  Pair p is rounds warp p and
+// schedule warp p + 4, which share a sub-partition: the schedule fills the issue slots that the rounds warp's
+// dependency chain leaves idle.
 // FS1, FS2: the forms (pk_sha256.cuh) of the schedule warp's additions for block 1 and block 2, `one` their
-// run-time 1 (with one pair per CTA the two blocks share one loop and FS1).  The rounds warp keeps the
-// compiler's form: its dependency chain sets the step time, and a multiply-add's longer latency there made
-// the four-pair chain slower (small-block key derivation 674 -> 718 us with every addition on the FMA pipe).
-// With four pairs each sub-partition runs a rounds warp and a schedule warp, whose two blocks differ:
+// run-time 1.  The rounds warp keeps the compiler's form: its dependency chain sets the step time, and a
+// multiply-add's longer latency there made the chain slower (small-block key derivation 674 -> 718 us with
+// every addition on the FMA pipe).  The schedule warp's two blocks differ:
 // block 1's schedule (k_{i-1} || d) can start only when k_{i-1} is published, and the rounds warp waits for
 // it after its 16th round, so it keeps the short-latency form; block 2's (c_i || padding) is made a step
 // ahead, off the critical path, and its additions go to the FMA pipe, where they do not compete with the
@@ -448,29 +439,25 @@ __device__ __forceinline__ void rounds16_kw(uint32_t v[8], const uint4 (*kw)[kCh
 // mad.lo by 2^(32-n): 4 and 6 cycles per warp instruction there) lost on either block (666-707 us): the
 // rounds warp's own multiply-adds queue behind them.  Block 2's first 16 words (K_t + W_t, set by
 // block2_head) and step 0's whole block 2, made before the loop, take FS1: 668 -> 654 us against FS2.
-template <int kPairs, int FS1, int FS2>
-__global__ void __launch_bounds__(2 * kChainLanes * kPairs, kPairs == 1 ? 15 : 4)
+constexpr int kChainPairs = 4;
+
+template <int FS1, int FS2>
+__global__ void __launch_bounds__(2 * kChainLanes * kChainPairs, 4)
 k_chain(const int64_t *key_off, const uint32_t *desc_idx,
         const uint8_t *digests, uint32_t R, uint32_t D, uint8_t *keys, uint32_t groups, uint32_t one) {
     extern __shared__ __align__(16) uint8_t chain_smem[];
     pk::pdl_wait(key_off, desc_idx, digests, keys);  // successor released at the last step (see k_chunk_digest)
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t pair = kPairs == 1 ? 0u : warp & (kPairs - 1);
-    const bool sched = kPairs == 1 ? warp == 1 : warp >= (uint32_t)kPairs;
+    const uint32_t pair = warp & (kChainPairs - 1);
+    const bool sched = warp >= (uint32_t)kChainPairs;
     ChainSmem &sm = reinterpret_cast<ChainSmem *>(chain_smem)[pair];
-    uint32_t group = blockIdx.x;
-    bool active = true;
-    if (kPairs > 1) {
-        const uint32_t g0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x);
-        const uint32_t g1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * groups / gridDim.x);
-        group = g0 + pair;
-        active = group < g1;
-    }
-    // named barriers of this pair (compile-time ids with one pair per CTA)
-    const int bar_s1 = kPairs == 1 ? 1 : 1 + 3 * (int)pair;  // block-1 schedule (first slice)
-    const int bar_s1b = kPairs == 1 ? 2 : 2 + 3 * (int)pair;  // block-1 schedule (second slice)
-    const int bar_b2 = kPairs == 1 ? 4 : -1;                  // block-2 schedule (four pairs: with bar_s1)
-    const int bar_k = kPairs == 1 ? 5 : 3 + 3 * (int)pair;   // k_i published
+    const uint32_t g0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x);
+    const uint32_t g1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * groups / gridDim.x);
+    const uint32_t group = g0 + pair;
+    const bool active = group < g1;
+    const int bar_s1 = 1 + 3 * (int)pair;   // block-1 schedule (first slice), and block 2 of the step
+    const int bar_s1b = 2 + 3 * (int)pair;  // block-1 schedule (second slice)
+    const int bar_k = 3 + 3 * (int)pair;    // k_i published
     const uint32_t r = group * kChainLanes + lane;
     int64_t a = 0, n = 0;
     uint32_t di = 0;
@@ -488,7 +475,7 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
     }
     if (nmax == 0) {  // uniform over the pair
         pk::pdl_launch_dependents();
-        if (kPairs > 1) __syncthreads();
+        __syncthreads();
         return;
     }
 
@@ -503,11 +490,6 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
     uint4 *kq = reinterpret_cast<uint4 *>(keys + 32ull * a);
 
     if (sched) {  // ---------------- schedule warp ----------------
-        // With one pair per CTA, one loop runs one copy of the 16-word schedule body for all six slices
-        // of a step (block-1 slices 1-3 of step i, then block-2 slices 1-3 of step i+1): the rounds warp
-        // on the next sub-partition slows down with the amount of distinct code this warp runs (per chain
-        // step, measured: 2206 ns with four unrolled copies, 2085 ns with one; 1950 ns with no schedule
-        // work at all).  With four pairs the two blocks have a loop each, in their own forms (FS1, FS2).
         // block 2 of step i: W = c_i (8 words) || 0x80000000, 0 x 6, 768; words 0..15 stored as K + W
         auto block2_head = [&](int64_t i, int buf, uint32_t w[16]) {
             if (i < n) {
@@ -535,7 +517,6 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
 #pragma unroll 1
             for (int q = 1; q < 4; ++q) schedule16<FS1>(w, sm.kw2[0], q, lane, one);
         }
-        if (kPairs == 1) bar_arrive(bar_b2);
 #pragma unroll 1
         for (int64_t i = 0; i < nmax; ++i) {
             if (i + 1 == nmax) pk::pdl_launch_dependents();
@@ -553,33 +534,19 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
                     w[4 * m + 2] = y.z;
                     w[4 * m + 3] = y.w;
                 }
-                if (kPairs == 1) bar_arrive(bar_b2);  // block-2 schedule of step i (made in the previous iteration)
             }
 #pragma unroll
             for (int j = 0; j < 8; ++j) w[8 + j] = dw[j];
             const int buf = (int)((i + 1) & 1);
-            if (kPairs == 1) {
-                const int slices = i + 1 < nmax ? 6 : 3;
+            schedule16<FS1>(w, sm.kw1, 1, lane, one);
+            bar_arrive(bar_s1);  // also: block 2 of step i ready
 #pragma unroll 1
-                for (int sl = 1; sl <= slices; ++sl) {
-                    if (sl == 4) block2_head(i + 1, buf, w);
-                    schedule16<FS1>(w, sl <= 3 ? sm.kw1 : sm.kw2[buf], sl <= 3 ? sl : sl - 3, lane, one);
-                    // constant barrier ids (a run-time id reserves all 16 named barriers)
-                    if (sl == 1) bar_arrive(1);
-                    else if (sl == 2) bar_arrive(2);
-                    else if (sl == 3) bar_arrive(3);
-                }
-            } else {
-                schedule16<FS1>(w, sm.kw1, 1, lane, one);
-                bar_arrive(bar_s1);  // also: block 2 of step i ready
+            for (int sl = 2; sl <= 3; ++sl) schedule16<FS1>(w, sm.kw1, sl, lane, one);
+            bar_arrive(bar_s1b);
+            if (i + 1 < nmax) {
+                block2_head(i + 1, buf, w);
 #pragma unroll 1
-                for (int sl = 2; sl <= 3; ++sl) schedule16<FS1>(w, sm.kw1, sl, lane, one);
-                bar_arrive(bar_s1b);
-                if (i + 1 < nmax) {
-                    block2_head(i + 1, buf, w);
-#pragma unroll 1
-                    for (int sl = 1; sl <= 3; ++sl) schedule16<FS2>(w, sm.kw2[buf], sl, lane, one);
-                }
+                for (int sl = 1; sl <= 3; ++sl) schedule16<FS2>(w, sm.kw2[buf], sl, lane, one);
             }
         }
         __syncthreads();  // stay resident until the rounds warp has consumed every phase
@@ -603,23 +570,13 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
             for (int j = 0; j < 8; ++j) pk::round_kw(a_, b_, c_, d_, e_, f_, g_, h_, kd[j]);
             v[0] = a_; v[1] = b_; v[2] = c_; v[3] = d_; v[4] = e_; v[5] = f_; v[6] = g_; v[7] = h_;
         }
-        if (kPairs == 1) {
-            bar_sync(1);
-            rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 1, lane, one);
-            bar_sync(2);
-            rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 2, lane, one);
-            bar_sync(3);
-            rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 3, lane, one);
-        } else {
-            bar_sync(bar_s1);
-            rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 1, lane, one);
-            bar_sync(bar_s1b);
-            rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 2, lane, one);
-            rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 3, lane, one);
-        }
+        bar_sync(bar_s1);
+        rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 1, lane, one);
+        bar_sync(bar_s1b);
+        rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 2, lane, one);
+        rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 3, lane, one);
         uint32_t st[8] = {PK_IV0 + v[0], PK_IV1 + v[1], PK_IV2 + v[2], PK_IV3 + v[3],
                           PK_IV4 + v[4], PK_IV5 + v[5], PK_IV6 + v[6], PK_IV7 + v[7]};
-        if (kPairs == 1) bar_sync(bar_b2);  // block-2 schedule of step i
         const uint4 (*kw2)[kChainLanes] = sm.kw2[i & 1];
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = st[j];
@@ -637,13 +594,286 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
     __syncthreads();
 }
 
+// ---------------------------------------------------------------------------
+// Chain with two lanes per request (split rounds and split schedule of
+// pk_sha256.cuh): 16 requests per pair of warps.  The chain of one request is
+// serial, so with few requests a step's latency is all that counts: a step is
+// 132 slots of about 24 cycles.  With one pair per CTA the two warps run on
+// different sub-partitions; with four, pair p is rounds warp p and schedule
+// warp p + 4, on one sub-partition.  The rounds are straight-line code (block 2
+// as a loop of 16 rounds: long-context key derivation 938 -> 1013 us), each
+// 16 words of K + W read while the 16 rounds before them run, and each barrier synced
+// some slots before the words it guards are needed.  The schedule warp's work
+// still costs the rounds warp about 8% (857 us with its arithmetic removed):
+// its shared-memory traffic is kept to 16-byte vectors (938 -> 924 us) and its
+// slices run one copy of the code.  Long-context key derivation (64 chains of
+// 512 steps) 1060 -> 925 us against one lane per request.
+// ---------------------------------------------------------------------------
+constexpr int kSplitReq = 16;                // requests per pair
+// A request's K+W row: its 32 even words, then (kSplitOdd) its 32 odd ones, each as 16-byte vectors.  The
+// schedule warp's lane stores four words of its parity at once; the row stride puts the vectors of a quarter
+// warp on distinct banks on either side.
+constexpr int kSplitOdd = 36;
+constexpr int kSplitRow = 72;
+struct SplitSmem {
+    uint32_t kw1[kSplitReq][kSplitRow];      // block-1 K+W, t = 16..63 used
+    uint32_t kw2[2][kSplitReq][kSplitRow];   // block-2 K+W, double-buffered by step parity
+    uint32_t zero[kSplitRow];                // the odd lanes' K+W
+    uint32_t kpub[kSplitReq][2][4];          // k_{i-1}: its even words, its odd words
+    uint32_t kpar[2][32];                    // K of the even and of the odd t
+};
+
+// K+W of rounds 16s .. 16s + 15
+__device__ __forceinline__ void ld16(uint32_t k[16], const uint32_t *row, int s) {
+#pragma unroll
+    for (int par = 0; par < 2; ++par) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const uint4 y = *reinterpret_cast<const uint4 *>(row + kSplitOdd * par + 8 * s + 4 * m);
+            k[8 * m + par] = y.x;
+            k[8 * m + 2 + par] = y.y;
+            k[8 * m + 4 + par] = y.z;
+            k[8 * m + 6 + par] = y.w;
+        }
+    }
+}
+
+template <int kPairs>
+__global__ void __launch_bounds__(64 * kPairs)
+k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *digests, uint32_t R, uint32_t D,
+              uint8_t *keys, uint32_t groups) {
+    extern __shared__ __align__(16) uint8_t chain_smem[];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t pair = kPairs == 1 ? 0u : warp & (kPairs - 1);
+    const bool sched = warp >= (uint32_t)kPairs;
+    const uint32_t q = lane >> 1, par = lane & 1;
+    SplitSmem &sm = reinterpret_cast<SplitSmem *>(chain_smem)[pair];
+    if (sched) {
+        sm.kpar[lane & 1][lane >> 1] = pk::kSha256K[lane];
+        sm.kpar[lane & 1][16 + (lane >> 1)] = pk::kSha256K[32 + lane];
+    } else {
+        for (int t = lane; t < kSplitRow; t += 32) sm.zero[t] = 0u;
+    }
+    __syncwarp();
+    pk::pdl_wait(key_off, desc_idx, digests, keys);  // successor released at the last step (see k_chunk_digest)
+    uint32_t group = blockIdx.x;
+    bool active = true;
+    if (kPairs > 1) {
+        const uint32_t g0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x);
+        const uint32_t g1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * groups / gridDim.x);
+        group = g0 + pair;
+        active = group < g1;
+    }
+    const int bar_s1 = 1 + 3 * (int)pair;   // block-1 schedule t = 16..31, and block 2 of the step
+    const int bar_s1b = 2 + 3 * (int)pair;  // block-1 schedule t = 32..63
+    const int bar_k = 3 + 3 * (int)pair;    // k_i published
+    const uint32_t r = group * kSplitReq + q;
+    int64_t a = 0, n = 0;
+    uint32_t di = 0;
+    if (active && r < R) {
+        a = key_off[r];
+        n = key_off[r + 1] - a;
+        di = desc_idx[r];
+        if (n < 0 || di >= D) n = 0;
+    }
+    int64_t nmax = n;  // identical in both warps of the pair: they cover the same requests
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int64_t x = __shfl_xor_sync(0xffffffffu, nmax, o);
+        nmax = x > nmax ? x : nmax;
+    }
+    if (nmax == 0) {  // uniform over the pair
+        pk::pdl_launch_dependents();
+        if (kPairs > 1) __syncthreads();
+        return;
+    }
+    uint32_t dw[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (n > 0) {
+        const uint4 *dq = reinterpret_cast<const uint4 *>(digests + 32ull * di);
+        const uint4 lo = __ldcg(dq), hi = __ldcg(dq + 1);
+        dw[0] = pk::bswap32(lo.x); dw[1] = pk::bswap32(lo.y); dw[2] = pk::bswap32(lo.z); dw[3] = pk::bswap32(lo.w);
+        dw[4] = pk::bswap32(hi.x); dw[5] = pk::bswap32(hi.y); dw[6] = pk::bswap32(hi.z); dw[7] = pk::bswap32(hi.w);
+    }
+    const pk::SplitLane l = pk::split_lane();
+    uint4 *kq = reinterpret_cast<uint4 *>(keys + 32ull * a);
+
+    if (sched) {  // ---------------- schedule warp ----------------
+        // c_i, loaded a step ahead of the schedule made from it
+        uint4 c_lo = make_uint4(0, 0, 0, 0), c_hi = c_lo;
+        auto fetch = [&](int64_t i) {
+            if (i < n) {
+                c_lo = __ldcg(kq + 2 * i);
+                c_hi = __ldcg(kq + 2 * i + 1);
+            }
+        };
+        // constant words t = 8..15 of block 2, in both buffers
+#pragma unroll
+        for (int i = 4; i < 8; ++i) {
+            const uint32_t t = 2 * i + par;
+            const uint32_t w = t == 8 ? 0x80000000u : t == 15 ? 96u * 8u : 0u;
+            sm.kw2[0][q][kSplitOdd * par + i] = sm.kpar[par][i] + w;
+            sm.kw2[1][q][kSplitOdd * par + i] = sm.kpar[par][i] + w;
+        }
+        uint32_t own[8], far[8], down[4], dfar[5];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {  // block 1: own[4 + j] = down[j], far[3 + j] = dfar[j]
+            down[j] = par ? dw[2 * j + 1] : dw[2 * j];
+            dfar[j + 1] = par ? (j < 3 ? dw[2 * j + 2] : 0u) : dw[2 * j + 1];
+        }
+        dfar[0] = dw[0];
+        // next 16 words t = 16s .. 16s + 15 of the ring -> K + W in row
+        auto slice = [&](uint32_t *row, int s) {
+            const uint4 *kp = reinterpret_cast<const uint4 *>(&sm.kpar[par][8 * s]);
+            const uint4 ka = kp[0], kb = kp[1];
+            uint4 *o = reinterpret_cast<uint4 *>(row + kSplitOdd * par + 8 * s);
+            pk::split_sched8(own, far, l);
+            o[0] = make_uint4(own[0] + ka.x, own[1] + ka.y, own[2] + ka.z, own[3] + ka.w);
+            o[1] = make_uint4(own[4] + kb.x, own[5] + kb.y, own[6] + kb.z, own[7] + kb.w);
+        };
+        auto block2 = [&](int64_t i, int buf) {  // words of block 2 of step i: c_i || 0x80000000, 0 x 6, 768
+            const uint32_t c[8] = {pk::bswap32(c_lo.x), pk::bswap32(c_lo.y), pk::bswap32(c_lo.z), pk::bswap32(c_lo.w),
+                                   pk::bswap32(c_hi.x), pk::bswap32(c_hi.y), pk::bswap32(c_hi.z), pk::bswap32(c_hi.w)};
+            fetch(i + 1);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                own[j] = par ? c[2 * j + 1] : c[2 * j];
+                far[j] = par ? (j < 3 ? c[2 * j + 2] : 0x80000000u) : c[2 * j + 1];
+            }
+            const uint4 ka = *reinterpret_cast<const uint4 *>(sm.kpar[par]);
+            *reinterpret_cast<uint4 *>(sm.kw2[buf][q] + kSplitOdd * par) =
+                make_uint4(own[0] + ka.x, own[1] + ka.y, own[2] + ka.z, own[3] + ka.w);
+            own[4] = par ? 0u : 0x80000000u;
+            own[5] = own[6] = 0u;
+            own[7] = par ? 96u * 8u : 0u;
+            far[4] = far[5] = far[6] = far[7] = 0u;
+        };
+        *reinterpret_cast<uint4 *>(sm.kpub[q][par]) = make_uint4(0, 0, 0, 0);  // k_{-1} = 0^32
+        __syncwarp();
+        fetch(0);
+        block2(0, 0);
+#pragma unroll 1
+        for (int s = 1; s < 4; ++s) slice(sm.kw2[0][q], s);
+#pragma unroll 1
+        for (int64_t i = 0; i < nmax; ++i) {
+            if (i + 1 == nmax) pk::pdl_launch_dependents();
+            if (i > 0) bar_sync(bar_k);  // k_{i-1} published; the rounds warp has finished step i-1
+            {
+                const uint4 x = *reinterpret_cast<const uint4 *>(sm.kpub[q][par]);
+                const uint4 y = *reinterpret_cast<const uint4 *>(sm.kpub[q][par ^ 1]);
+                own[0] = x.x; own[1] = x.y; own[2] = x.z; own[3] = x.w;
+                far[0] = par ? y.y : y.x;
+                far[1] = par ? y.z : y.y;
+                far[2] = par ? y.w : y.z;
+                far[3] = par ? dfar[0] : y.w;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    own[4 + j] = down[j];
+                    far[4 + j] = dfar[j + 1];
+                }
+            }
+            const int buf = (int)((i + 1) & 1);
+            const int slices = i + 1 < nmax ? 6 : 3;
+#pragma unroll 1
+            for (int s = 1; s <= slices; ++s) {  // one copy of the slice body
+                if (s == 4) block2(i + 1, buf);
+                slice(s <= 3 ? sm.kw1[q] : sm.kw2[buf][q], s <= 3 ? s : s - 3);
+                if (s == 1) bar_arrive(bar_s1);
+                else if (s == 3) bar_arrive(bar_s1b);
+            }
+        }
+        __syncthreads();  // stay resident until the rounds warp has consumed every phase
+        return;
+    }
+
+    // ---------------- rounds warp ----------------
+    const uint32_t iv[4] = {l.even ? PK_IV4 : PK_IV0, l.even ? PK_IV5 : PK_IV1, l.even ? PK_IV6 : PK_IV2,
+                            l.even ? PK_IV7 : PK_IV3};
+    const uint32_t mA = l.even ? 1u : 0u;
+    uint32_t kc[8], kd[8];  // K_t, t = 0..7, and K_t + d_{t-8}, t = 8..15, in the even lanes
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        kc[j] = l.even ? pk::kSha256K[j] : 0u;
+        kd[j] = l.even ? pk::kSha256K[8 + j] + dw[j] : 0u;
+    }
+    const uint32_t *row1 = l.even ? sm.kw1[q] : sm.zero;
+    uint32_t p[4] = {0, 0, 0, 0};  // k_{-1} = 0^32 (even lane: words 4..7, odd lane: words 0..3)
+    __syncwarp();
+#pragma unroll 1
+    for (int64_t i = 0; i < nmax; ++i) {
+        if (i + 1 == nmax) pk::pdl_launch_dependents();
+        uint32_t k[16], kn[16], cd[2];
+        uint32_t st[4] = {iv[0], iv[1], iv[2], iv[3]};
+        pk::SplitState v;
+        pk::split_start(v, l, st, PK_IV2, PK_IV3);
+        // block 1, rounds 0..15: W = k_{i-1} || d
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t o = __shfl_xor_sync(0xffffffffu, p[j], 1);
+            k[j] = pk::mad1(o, mA, kc[j]);
+            k[4 + j] = pk::mad1(p[j], mA, kc[4 + j]);
+        }
+        pk::split_slot<true>(v, l, k[0], st[1]);
+        pk::split_slot<true>(v, l, k[1], st[0]);
+#pragma unroll
+        for (int j = 2; j < 8; ++j) pk::split_slot(v, l, k[j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pk::split_slot(v, l, kd[j]);
+        bar_sync(bar_s1);
+        ld16(kn, row1, 1);
+#pragma unroll
+        for (int j = 4; j < 8; ++j) pk::split_slot(v, l, kd[j]);
+#pragma unroll
+        for (int j = 0; j < 12; ++j) pk::split_slot(v, l, kn[j]);
+        bar_sync(bar_s1b);
+        ld16(k, row1, 2);
+#pragma unroll
+        for (int j = 12; j < 16; ++j) pk::split_slot(v, l, kn[j]);
+        ld16(kn, row1, 3);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pk::split_slot(v, l, k[j]);
+        const uint32_t *r2 = l.even ? sm.kw2[i & 1][q] : sm.zero;
+        ld16(k, r2, 0);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pk::split_slot(v, l, kn[j]);
+        pk::split_end(v, l, st, cd);
+        // block 2
+        pk::split_start(v, l, st, PK_IV2 + cd[0], PK_IV3 + cd[1]);
+        ld16(kn, r2, 1);
+        pk::split_slot<true>(v, l, k[0], st[1]);
+        pk::split_slot<true>(v, l, k[1], st[0]);
+#pragma unroll
+        for (int j = 2; j < 16; ++j) pk::split_slot(v, l, k[j]);
+        ld16(k, r2, 2);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pk::split_slot(v, l, kn[j]);
+        ld16(kn, r2, 3);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pk::split_slot(v, l, k[j]);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) pk::split_slot(v, l, kn[j]);
+        pk::split_end(v, l, st, cd);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) p[j] = st[j];
+        const uint32_t half = l.even ? 1u : 0u;  // the even lane holds the second half of the key
+        if (i + 1 < nmax) {
+            *reinterpret_cast<uint2 *>(&sm.kpub[q][0][2 * half]) = make_uint2(p[0], p[2]);
+            *reinterpret_cast<uint2 *>(&sm.kpub[q][1][2 * half]) = make_uint2(p[1], p[3]);
+            bar_arrive(bar_k);
+        }
+        if (i < n)
+            kq[2 * i + half] = make_uint4(pk::bswap32(p[0]), pk::bswap32(p[1]), pk::bswap32(p[2]), pk::bswap32(p[3]));
+    }
+    __syncthreads();
+}
+
 unsigned grid_for(uint64_t n, unsigned block) { return (unsigned)((n + block - 1) / block); }
 
 // Shared memory of the four-pair chain CTA: its four ChainSmem (100 KiB), padded past half of an SM's
 // shared memory so that no SM holds two of these CTAs (the launch becomes resident while the chunk digests
 // drain, and would otherwise stack CTAs on the SMs that free up first).
 constexpr size_t kChainPackedSmem = 116 * 1024;
-static_assert(kChainPackedSmem >= 4 * sizeof(ChainSmem), "four pairs fit");
+constexpr size_t kChainHalfSmem = 76 * 1024;  // past a third: at most two CTAs per SM
+static_assert(kChainPackedSmem >= kChainPairs * sizeof(ChainSmem), "four pairs fit");
 
 // Raise the four-pair chain CTA's shared-memory limit once per device.
 cudaError_t chain_packed_attr() {
@@ -655,8 +885,28 @@ cudaError_t chain_packed_attr() {
     if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!done[dev]) {
-        e = cudaFuncSetAttribute(k_chain<4, pk::kAddsPlain, pk::kAddsFma>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(k_chain<pk::kAddsPlain, pk::kAddsFma>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kChainPackedSmem);
+        if (e != cudaSuccess) return e;
+        done[dev] = true;
+    }
+    return cudaSuccess;
+}
+
+static_assert(kChainPackedSmem >= 4 * sizeof(SplitSmem), "four split pairs fit");
+// Raise the two-lane chain CTAs' shared-memory limit once per device.
+cudaError_t chain_split_attr() {
+    static std::mutex mu;
+    static bool done[256] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!done[dev]) {
+        e = cudaFuncSetAttribute(k_chain_split<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_chain_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
         if (e != cudaSuccess) return e;
         done[dev] = true;
     }
@@ -716,18 +966,32 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
             : pk_launch(k_chunk_digest<pk::kAddsPlain>, grid, kDigestBlock, s, tokens, tok_off,
                         (const int64_t *)key_off, R, C, pad, keys, dw, one);
     if (e != cudaSuccess) return e;
-    // Chains: one pair per CTA while the groups of 32 requests fit one per SM; four pairs per CTA (one CTA
-    // per SM, each pair on its own sub-partition) for more groups.
-    const uint32_t groups = grid_for(R, kChainLanes);
-    if (ctx->sm_count == 0 || groups <= ctx->sm_count) {
-        e = pk_launch_smem(k_chain<1, pk::kAddsPlain, pk::kAddsPlain>, groups, 2 * kChainLanes, sizeof(ChainSmem), s,
-                           (const int64_t *)key_off, desc_idx, (const uint8_t *)digests, R, D, keys, groups, one);
-    } else {
-        e = chain_packed_attr();
-        const uint32_t grid = groups <= 4 * ctx->sm_count ? ctx->sm_count : grid_for(groups, 4);
+    // Chains, by pairs of 16 requests per SM (rounded up).  Key derivation of R prompts of 32 chunks of 16
+    // tokens, measured, in us, for: two lanes per request, one pair per CTA | four pairs per CTA | one lane per
+    // request:  R = 2432 (1 pair per SM) 77 | 94 | 112;  4864 (2) 87 | 103 | 121;  7296 (3) 134 | 114 | 131;
+    // 9728 (4) 145 | 126 | 143;  11000 (5) 197 | 201 | 148;  16384 (7) 263 | 225 | 172.
+    const uint32_t groups = grid_for(R, kSplitReq);
+    const uint32_t sms = ctx->sm_count;
+    const uint32_t per_sm = sms ? grid_for(groups, sms) : 1;
+    if (per_sm <= 2) {
+        // Shared memory padded so that no SM takes more than its share of the CTAs (R = 4864 without: 123 us).
+        const size_t smem = per_sm == 1 ? kChainPackedSmem : kChainHalfSmem;
+        e = chain_split_attr();
         if (e == cudaSuccess)
-            e = pk_launch_smem(k_chain<4, pk::kAddsPlain, pk::kAddsFma>, grid, 8 * kChainLanes, kChainPackedSmem, s,
-                               (const int64_t *)key_off, desc_idx, (const uint8_t *)digests, R, D, keys, groups, one);
+            e = pk_launch_smem(k_chain_split<1>, groups, 64, smem, s, (const int64_t *)key_off, desc_idx,
+                               (const uint8_t *)digests, R, D, keys, groups);
+    } else if (per_sm <= 4) {
+        e = chain_split_attr();
+        if (e == cudaSuccess)
+            e = pk_launch_smem(k_chain_split<4>, sms, 256, kChainPackedSmem, s, (const int64_t *)key_off, desc_idx,
+                               (const uint8_t *)digests, R, D, keys, groups);
+    } else {
+        const uint32_t g32 = grid_for(R, kChainLanes);
+        e = chain_packed_attr();
+        const uint32_t grid = g32 <= 4 * sms ? sms : grid_for(g32, 4);
+        if (e == cudaSuccess)
+            e = pk_launch_smem(k_chain<pk::kAddsPlain, pk::kAddsFma>, grid, 8 * kChainLanes, kChainPackedSmem, s,
+                               (const int64_t *)key_off, desc_idx, (const uint8_t *)digests, R, D, keys, g32, one);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

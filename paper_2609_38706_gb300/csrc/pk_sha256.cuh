@@ -306,6 +306,116 @@ __device__ __forceinline__ void compress_kw(uint32_t st[8], const uint32_t *__re
     st[6] = add2<F>(st[6], g, one); st[7] = add2<F>(st[7], h, one);
 }
 
+// ---------------------------------------------------------------------------
+// Split rounds: two lanes per message.  The rounds are two recurrences,
+//   e_{t+1} = a_{t-3} + e_{t-3} + S1(e_t) + Ch(e_t, e_{t-1}, e_{t-2}) + K_t + W_t
+//   a_{t+1} = e_{t+1} - a_{t-3} + S0(a_t) + Maj(a_t, a_{t-1}, a_{t-2})
+// of one form, out = rotations of x0 + select(x0; x1, x2) + (+-x3 + kw) + q,
+// so that one instruction stream serves both: the even lane of a pair holds
+// e..h (x0..x3), the odd lane a..d, and q is the other lane's output of two
+// slots before.  The odd lane runs two rounds behind the even one: e_{t+1}
+// reaches it two slots after it was made, just when a_{t+1} needs it, and
+// a_{t-3} reaches the even lane two slots after it was made, just when e_{t+1}
+// needs it, so that neither lane waits for a shuffle.  A lone warp is bound by
+// the dependency chain of a round (three rotations issued two cycles apart on
+// the half-rate ALU, a 3-input xor, a 3-input add: 20.7 cycles, measured), not
+// by throughput; one lane per message runs two such chains and all their
+// operations through the one pipe (10 logic operations and the adds).  Measured
+// on GB300, cycles per 64 rounds of a lone warp with K + W in shared memory: 2637
+// with one lane per message (round_kw), 1605 with two; with two warps per SM
+// sub-partition 2854 for 2 x 16 messages, so a full sub-partition is better
+// served by one lane per message.
+// The select is written over P and Q, made a slot ahead of their use:
+// Ch = e ? f : g, Maj = a ? (b | c) : (b & c).
+// ---------------------------------------------------------------------------
+struct SplitLane {
+    uint32_t r1, r2, r3;  // rotations of S1 (even lane) or S0 (odd lane)
+    uint32_t maj;         // all ones in the odd lane
+    uint32_t sign;        // x3 enters with +1 (even lane) or -1 (odd lane)
+    bool even;
+};
+
+__device__ __forceinline__ SplitLane split_lane() {
+    const bool even = (threadIdx.x & 1) == 0;
+    return even ? SplitLane{6, 11, 25, 0u, 1u, true} : SplitLane{2, 13, 22, 0xffffffffu, 0xffffffffu, false};
+}
+
+struct SplitState {
+    uint32_t x[4];    // e..h or a..d, the newest first
+    uint32_t q0, q1;  // the other lane's outputs for this slot and the next
+    uint32_t P, Q;    // the select's operands for this slot
+};
+
+// One slot: round t in the even lane, round t - 2 in the odd lane.  kw = K_t + W_t
+// in the even lane, 0 in the odd lane.  kForced (slots 0 and 1 of a compression):
+// the odd lane, whose rounds begin at slot 2, takes `forced` instead.
+template <bool kForced = false>
+__device__ __forceinline__ void split_slot(SplitState &v, const SplitLane &l, uint32_t kw, uint32_t forced = 0u) {
+    const uint32_t x0 = v.x[0];
+    const uint32_t S = __funnelshift_r(x0, x0, l.r1) ^ __funnelshift_r(x0, x0, l.r2) ^ __funnelshift_r(x0, x0, l.r3);
+    const uint32_t sel = (x0 & v.P) | (~x0 & v.Q);
+    uint32_t z;
+    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(z) : "r"(v.x[3]), "r"(l.sign), "r"(kw));
+    uint32_t X = v.q0 + z;
+    asm("" : "+r"(X));  // keep the late sum one 3-input add
+    uint32_t out = S + sel + X;
+    if (kForced) out = l.even ? out : forced;
+    v.P = x0 | (v.x[1] & l.maj);
+    v.Q = v.x[1] & (x0 | ~l.maj);
+    v.q0 = v.q1;
+    v.q1 = __shfl_xor_sync(0xffffffffu, out, 1);
+    v.x[3] = v.x[2];
+    v.x[2] = v.x[1];
+    v.x[1] = x0;
+    v.x[0] = out;
+}
+
+// Start of a compression from the state st (e..h / a..d); c, d: the even lane's
+// copies of the state's third and fourth word.  Slots 0 and 1 are split_slot<true>
+// with forced = st[1] and st[0].
+__device__ __forceinline__ void split_start(SplitState &v, const SplitLane &l, const uint32_t st[4], uint32_t c,
+                                            uint32_t d) {
+    v.x[0] = l.even ? st[0] : st[2];
+    v.x[1] = l.even ? st[1] : st[3];
+    v.x[2] = st[2];
+    v.x[3] = st[3];
+    v.q0 = d;
+    v.q1 = c;
+    v.P = v.x[1] | (v.x[2] & l.maj);
+    v.Q = v.x[2] & (v.x[1] | ~l.maj);
+}
+
+// After slot 63: the odd lane's last two rounds, then st += the final state.
+// c_d[0], c_d[1]: in the even lane, the final state's third and fourth word
+// (before the addition), for the next compression's start.
+__device__ __forceinline__ void split_end(SplitState &v, const SplitLane &l, uint32_t st[4], uint32_t c_d[2]) {
+    const uint32_t e0 = v.x[0], e1 = v.x[1], e2 = v.x[2], e3 = v.x[3];
+    c_d[1] = v.q0;  // a_61
+    c_d[0] = v.q1;  // a_62
+    split_slot(v, l, 0u);
+    split_slot(v, l, 0u);
+    st[0] += l.even ? e0 : v.x[0];
+    st[1] += l.even ? e1 : v.x[1];
+    st[2] += l.even ? e2 : v.x[2];
+    st[3] += l.even ? e3 : v.x[3];
+}
+
+// Message schedule over the same two lanes: the even lane holds the even
+// words (own[i] = W_{2i}), the odd lane the odd ones (own[i] = W_{2i+1}), and
+// far[i] the other lane's word between them and the next (even lane: W_{2i+1},
+// odd lane: W_{2i+2}).  One call makes the next eight words of each lane in
+// place.  far[7] is not read before the first step has delivered it, one step after the others.
+__device__ __forceinline__ void split_sched8(uint32_t own[8], uint32_t far[8], const SplitLane &l) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t prev = own[(i + 7) & 7];
+        const uint32_t early = far[(i + 4) & 7] + own[i] + small_s0(far[i]);
+        const uint32_t w = early + small_s1(prev);
+        own[i] = w;
+        far[(i + 7) & 7] = __shfl_xor_sync(0xffffffffu, l.even ? w : prev, 1);
+    }
+}
+
 }  // namespace pk
 #endif
 
