@@ -640,7 +640,8 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
 // still costs the rounds warp about 8% (857 us with its arithmetic removed):
 // its shared-memory traffic is kept to 16-byte vectors (938 -> 924 us) and its
 // slices run one copy of the code.  Long-context key derivation (64 chains of
-// 512 steps) 1060 -> 925 us against one lane per request.
+// 512 steps) 1060 -> 925 us against one lane per request, 865 us with the
+// select's P on the FMA pipe.
 // ---------------------------------------------------------------------------
 constexpr int kSplitReq = 16;                // requests per pair
 // A request's K+W row: its 32 even words, then (kSplitOdd) its 32 odd ones, each as 16-byte vectors.  The
@@ -674,7 +675,7 @@ __device__ __forceinline__ void ld16(uint32_t k[16], const uint32_t *row, int s)
 template <int kPairs>
 __global__ void __launch_bounds__(64 * kPairs)
 k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *digests, uint32_t R, uint32_t D,
-              uint8_t *keys, uint32_t groups) {
+              uint8_t *keys, uint32_t groups, uint32_t one) {
     extern __shared__ __align__(16) uint8_t chain_smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t pair = kPairs == 1 ? 0u : warp & (kPairs - 1);
@@ -727,7 +728,7 @@ k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *d
         dw[0] = pk::bswap32(lo.x); dw[1] = pk::bswap32(lo.y); dw[2] = pk::bswap32(lo.z); dw[3] = pk::bswap32(lo.w);
         dw[4] = pk::bswap32(hi.x); dw[5] = pk::bswap32(hi.y); dw[6] = pk::bswap32(hi.z); dw[7] = pk::bswap32(hi.w);
     }
-    const pk::SplitLane l = pk::split_lane();
+    const pk::SplitLane l = pk::split_lane(one);
     uint4 *kq = reinterpret_cast<uint4 *>(keys + 32ull * a);
 
     if (sched) {  // ---------------- schedule warp ----------------
@@ -1012,12 +1013,12 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
         e = chain_split_attr();
         if (e == cudaSuccess)
             e = pk_launch_smem(k_chain_split<1>, groups, 64, smem, s, (const int64_t *)key_off, desc_idx,
-                               (const uint8_t *)digests, R, D, keys, groups);
+                               (const uint8_t *)digests, R, D, keys, groups, one);
     } else if (per_sm <= 4) {
         e = chain_split_attr();
         if (e == cudaSuccess)
             e = pk_launch_smem(k_chain_split<4>, sms, 256, kChainPackedSmem, s, (const int64_t *)key_off, desc_idx,
-                               (const uint8_t *)digests, R, D, keys, groups);
+                               (const uint8_t *)digests, R, D, keys, groups, one);
     } else {
         const uint32_t g32 = grid_for(R, kChainLanes);
         e = chain_packed_attr();

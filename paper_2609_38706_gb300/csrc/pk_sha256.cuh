@@ -322,8 +322,8 @@ __device__ __forceinline__ void compress_kw(uint32_t st[8], const uint32_t *__re
 // by throughput; one lane per message runs two such chains and all their
 // operations through the one pipe (10 logic operations and the adds).  Measured
 // on GB300, cycles per 64 rounds of a lone warp with K + W in shared memory: 2637
-// with one lane per message (round_kw), 1605 with two; with two warps per SM
-// sub-partition 2854 for 2 x 16 messages, so a full sub-partition is better
+// with one lane per message (round_kw), 1488 with two; with two warps per SM
+// sub-partition 2520 for 2 x 16 messages, so a full sub-partition is better
 // served by one lane per message.
 // The select is written over P and Q, made a slot ahead of their use:
 // Ch = e ? f : g, Maj = a ? (b | c) : (b & c).
@@ -332,12 +332,14 @@ struct SplitLane {
     uint32_t r1, r2, r3;  // rotations of S1 (even lane) or S0 (odd lane)
     uint32_t maj;         // all ones in the odd lane
     uint32_t sign;        // x3 enters with +1 (even lane) or -1 (odd lane)
+    uint32_t one, minus;  // a run-time 1 and -1 (see mad1)
     bool even;
 };
 
-__device__ __forceinline__ SplitLane split_lane() {
+__device__ __forceinline__ SplitLane split_lane(uint32_t one) {
     const bool even = (threadIdx.x & 1) == 0;
-    return even ? SplitLane{6, 11, 25, 0u, 1u, true} : SplitLane{2, 13, 22, 0xffffffffu, 0xffffffffu, false};
+    return even ? SplitLane{6, 11, 25, 0u, 1u, one, 0u - one, true}
+                : SplitLane{2, 13, 22, 0xffffffffu, 0xffffffffu, one, 0u - one, false};
 }
 
 struct SplitState {
@@ -345,6 +347,13 @@ struct SplitState {
     uint32_t q0, q1;  // the other lane's outputs for this slot and the next
     uint32_t P, Q;    // the select's operands for this slot
 };
+
+// The select's operands for a slot with x1 = b and x2 = c: Q = c or b & c, and P = b or b | c as (b + c) - Q on
+// the FMA pipe (a lone warp's 64 rounds 1598 cycles with P as a logic operation, 1488 so).
+__device__ __forceinline__ void split_select(SplitState &v, const SplitLane &l, uint32_t b, uint32_t c) {
+    v.Q = c & (b | ~l.maj);
+    v.P = mad1(v.Q, l.minus, mad1(c, l.one, b));
+}
 
 // One slot: round t in the even lane, round t - 2 in the odd lane.  kw = K_t + W_t
 // in the even lane, 0 in the odd lane.  kForced (slots 0 and 1 of a compression):
@@ -354,14 +363,11 @@ __device__ __forceinline__ void split_slot(SplitState &v, const SplitLane &l, ui
     const uint32_t x0 = v.x[0];
     const uint32_t S = __funnelshift_r(x0, x0, l.r1) ^ __funnelshift_r(x0, x0, l.r2) ^ __funnelshift_r(x0, x0, l.r3);
     const uint32_t sel = (x0 & v.P) | (~x0 & v.Q);
-    uint32_t z;
-    asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(z) : "r"(v.x[3]), "r"(l.sign), "r"(kw));
-    uint32_t X = v.q0 + z;
+    uint32_t X = v.q0 + mad1(v.x[3], l.sign, kw);
     asm("" : "+r"(X));  // keep the late sum one 3-input add
     uint32_t out = S + sel + X;
     if (kForced) out = l.even ? out : forced;
-    v.P = x0 | (v.x[1] & l.maj);
-    v.Q = v.x[1] & (x0 | ~l.maj);
+    split_select(v, l, x0, v.x[1]);
     v.q0 = v.q1;
     v.q1 = __shfl_xor_sync(0xffffffffu, out, 1);
     v.x[3] = v.x[2];
@@ -381,8 +387,7 @@ __device__ __forceinline__ void split_start(SplitState &v, const SplitLane &l, c
     v.x[3] = st[3];
     v.q0 = d;
     v.q1 = c;
-    v.P = v.x[1] | (v.x[2] & l.maj);
-    v.Q = v.x[2] & (v.x[1] | ~l.maj);
+    split_select(v, l, v.x[1], v.x[2]);
 }
 
 // After slot 63: the odd lane's last two rounds, then st += the final state.
