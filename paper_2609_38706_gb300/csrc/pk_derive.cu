@@ -632,8 +632,9 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
 // pk_sha256.cuh): 16 requests per pair of warps.  The chain of one request is
 // serial, so with few requests a step's latency is all that counts: a step is
 // 132 slots of about 24 cycles.  With one pair per CTA the two warps run on
-// different sub-partitions; with four, pair p is rounds warp p and schedule
-// warp p + 4, on one sub-partition.  The rounds are straight-line code (block 2
+// different sub-partitions; with three, the rounds warps have a sub-partition
+// each and the schedule warps share the fourth; with four, pair p is rounds
+// warp p and schedule warp p + 4, on one sub-partition.  The rounds are straight-line code (block 2
 // as a loop of 16 rounds: long-context key derivation 938 -> 1013 us), each
 // 16 words of K + W read while the 16 rounds before them run, and each barrier synced
 // some slots before the words it guards are needed.  The schedule warp's work
@@ -672,14 +673,22 @@ __device__ __forceinline__ void ld16(uint32_t k[16], const uint32_t *row, int s)
     }
 }
 
+// Warps of a CTA of kPairs pairs: with three pairs the rounds warps are warps 0, 1, 2 and the schedule warps 3, 7,
+// 11 (warps 4-6 and 8-10 do nothing).
+constexpr int split_warps(int pairs) { return pairs == 3 ? 12 : 2 * pairs; }
+
 template <int kPairs>
-__global__ void __launch_bounds__(64 * kPairs)
+__global__ void __launch_bounds__(32 * split_warps(kPairs))
 k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *digests, uint32_t R, uint32_t D,
               uint8_t *keys, uint32_t groups, uint32_t one) {
     extern __shared__ __align__(16) uint8_t chain_smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t pair = kPairs == 1 ? 0u : warp & (kPairs - 1);
-    const bool sched = warp >= (uint32_t)kPairs;
+    const bool sched = kPairs == 3 ? (warp & 3) == 3 : warp >= (uint32_t)kPairs;
+    const uint32_t pair = kPairs == 3 && sched ? warp >> 2 : kPairs == 4 ? warp & 3 : kPairs == 1 ? 0u : warp;
+    if (kPairs == 3 && pair >= 3) {
+        __syncthreads();
+        return;
+    }
     const uint32_t q = lane >> 1, par = lane & 1;
     SplitSmem &sm = reinterpret_cast<SplitSmem *>(chain_smem)[pair];
     if (sched) {
@@ -940,6 +949,8 @@ cudaError_t chain_split_attr() {
     if (!done[dev]) {
         e = cudaFuncSetAttribute(k_chain_split<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
         if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_chain_split<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
+        if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_chain_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
         if (e != cudaSuccess) return e;
         done[dev] = true;
@@ -1001,9 +1012,9 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
                         (const int64_t *)key_off, R, C, pad, keys, dw, one);
     if (e != cudaSuccess) return e;
     // Chains, by pairs of 16 requests per SM (rounded up).  Key derivation of R prompts of 32 chunks of 16
-    // tokens, measured, in us, for: two lanes per request, one pair per CTA | four pairs per CTA | one lane per
-    // request:  R = 2432 (1 pair per SM) 77 | 94 | 112;  4864 (2) 87 | 103 | 121;  7296 (3) 134 | 114 | 131;
-    // 9728 (4) 145 | 126 | 143;  11000 (5) 197 | 201 | 148;  16384 (7) 263 | 225 | 172.
+    // tokens, measured, in us, for: two lanes per request, one pair per CTA | three | four | one lane per request:
+    // R = 2432 (1 pair per SM) 73 | - | 94 | 112;  4864 (2) 83 | - | 103 | 121;  7296 (3) 134 | 110 | 114 | 131;
+    // 9728 (4) 145 | - | 126 | 143;  11000 (5) 197 | - | 201 | 148;  16384 (7) 263 | - | 225 | 172.
     const uint32_t groups = grid_for(R, kSplitReq);
     const uint32_t sms = ctx->sm_count;
     const uint32_t per_sm = sms ? grid_for(groups, sms) : 1;
@@ -1014,10 +1025,15 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
         if (e == cudaSuccess)
             e = pk_launch_smem(k_chain_split<1>, groups, 64, smem, s, (const int64_t *)key_off, desc_idx,
                                (const uint8_t *)digests, R, D, keys, groups, one);
-    } else if (per_sm <= 4) {
+    } else if (per_sm == 3) {
         e = chain_split_attr();
         if (e == cudaSuccess)
-            e = pk_launch_smem(k_chain_split<4>, sms, 256, kChainPackedSmem, s, (const int64_t *)key_off, desc_idx,
+            e = pk_launch_smem(k_chain_split<3>, sms, 32 * split_warps(3), kChainPackedSmem, s, (const int64_t *)key_off,
+                               desc_idx, (const uint8_t *)digests, R, D, keys, groups, one);
+    } else if (per_sm == 4) {
+        e = chain_split_attr();
+        if (e == cudaSuccess)
+            e = pk_launch_smem(k_chain_split<4>, sms, 32 * split_warps(4), kChainPackedSmem, s, (const int64_t *)key_off, desc_idx,
                                (const uint8_t *)digests, R, D, keys, groups, one);
     } else {
         const uint32_t g32 = grid_for(R, kChainLanes);

@@ -1,5 +1,5 @@
-"""The chain's layouts (two lanes per request with one or four pairs of warps per CTA, one lane per request) at the
-edges of their ranges: requests per pair (16), pairs per SM (2, 4), uneven and empty requests."""
+"""The chain's layouts (two lanes per request with one, three or four pairs of warps per CTA, one lane per request) at the
+edges of their ranges: requests per pair (16), pairs per SM (2, 3, 4), uneven and empty requests."""
 import numpy as np
 import pytest
 import torch
@@ -35,7 +35,7 @@ def test_few_requests(R, max_chunks):
     check(R, 4, max_chunks, 100 * R + max_chunks)
 
 
-@pytest.mark.parametrize("pairs_per_sm", [1, 2, 4])
+@pytest.mark.parametrize("pairs_per_sm", [1, 2, 3, 4])
 @pytest.mark.parametrize("past", [-1, 0, 1])
 def test_layout_boundaries(pairs_per_sm, past):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
