@@ -16,21 +16,30 @@
 // bounded grid barriers:
 //   1. every CTA reads the entry count and returns at once when it is within
 //      the budget (the common step costs one short launch);
-//   2. gather: one bit per entry (occupied), and the stamp and slot of every
-//      occupied entry compacted into scratch, with the smallest and largest
-//      stamp;
-//   3. radix select of v over the gathered stamps, 8 bits per pass from the
-//      highest byte in which the smallest and largest stamp differ (the bytes
-//      above are common to all); each pass is a shared-memory histogram of
-//      the candidates with warp-aggregated increments, and every CTA then
-//      picks the same bucket;
-//   4. the slots of the gathered entries with stamp <= v are compacted into
-//      the output (one atomic per warp), and the table is compacted in place,
-//      one thread per cluster (maximal run of occupied entries, from the
-//      bitmap of phase 2): in probe order, an evicted entry is cleared; a kept
-//      entry moves to the first empty position between its home and its own,
-//      so that every kept key stays reachable by linear probing.  Clusters
-//      are disjoint, so no two threads touch the same entry.
+//   2. gather: one bit per entry (occupied), one byte with its distance from
+//      home, the numbers of entries with and without a stamp, the range of
+//      the stamps, and a histogram of their age in store calls;
+//   3. the threshold v: the age histogram gives the call in which the last
+//      entry to go was used; if every entry of that call and the calls before
+//      it goes, v is known (a store that evicts whole batches, the common
+//      case).  Otherwise the stamps of that call are split by their key
+//      index, 8 bits per pass over the stamp array, until the entries to go
+//      end with a bucket;
+//   4. every position with a stamp <= v goes into an evicted bitmap and its
+//      slot into the output (buffered in shared memory), and the table is
+//      compacted in place, one thread per cluster (maximal run of occupied
+//      entries, from the bitmap of phase 2): in probe order, an evicted entry
+//      is cleared; a kept entry moves to the first empty position between its
+//      home and its own, so that every kept key stays reachable by linear
+//      probing.  Clusters are disjoint, so no two threads touch the same entry.
+// Every phase but the last streams over the table or the stamps and is bound
+// by loads in flight: two CTAs of 512 threads per SM, four positions per
+// thread (a bulk prefetch into L2 of the next iteration changed nothing).
+// 2^22 entries, 1.84 M stored, 262,144 evicted (one call's): 190 -> 86 us
+// (gather 37, threshold 5, bitmap and slots 17, compaction 26), against
+// compacting stamps and slots into a list, selecting over it in 5 passes and
+// two more passes for the slots and the bitmap, with one CTA per SM.
+// 2^14 entries, 512 of 5,120 evicted: 54 -> 18 us.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -41,16 +50,22 @@
 namespace {
 
 constexpr uint32_t kEvThreads = 512;
+constexpr uint32_t kEvBlocks = 2;  // CTAs per SM
+constexpr uint32_t kEvRows = 512;  // table entries per CTA below which no further CTA is launched
+constexpr uint32_t kPasses = 7;    // histogram rows of the passes within a call, used in turn
 constexpr uint32_t kSpinLimit = 1u << 23;  // x ~100 ns: a barrier gives up after about a second
 
 struct EvictHeader {  // zeroed by the host before every launch
-    unsigned int arrive;
-    unsigned int gen;
-    unsigned long long n;          // entries gathered
-    unsigned long long n_evicted;  // entries removed
-    unsigned long long inv_min;    // ~(smallest stamp gathered)
-    unsigned long long max;        // largest stamp gathered
-    unsigned int hist[8][256];
+    unsigned int arrive;             // CTAs that have arrived at the grid barriers so far
+    unsigned int unused;
+    unsigned long long n_stamped;    // entries with a stamp
+    unsigned long long n_unstamped;  // entries without (stamp 0)
+    unsigned long long n_evicted;    // entries removed
+    unsigned long long inv_min;      // ~(smallest non-zero stamp)
+    unsigned long long max;          // largest stamp
+    unsigned int max_index;          // largest key index (low half) of a stamp
+    unsigned int age[256];           // stamped entries by age in calls, 255: that and older
+    unsigned int hist[kPasses][256];
 };
 constexpr uint64_t kHeaderBytes = (sizeof(EvictHeader) + 255) & ~255ull;
 
@@ -72,74 +87,85 @@ struct BarrierBound {
     uint32_t withheld_cta;
 };
 
-// Grid-wide barrier with a bounded wait.  Returns false (in every thread of
-// the CTA) when the wait gave up; the status word then holds PK_ERR_TIMEOUT.
-// A withheld CTA returns false without arriving.
-__device__ bool grid_sync(EvictHeader *h, int32_t *status, const BarrierBound &bb) {
+// Grid-wide barrier number `k` (from 0) of the launch, with a bounded wait: a
+// barrier is passed once (k + 1) x gridDim arrivals are counted, so that
+// arriving and seeing the last arrival take one round trip to L2 each (a
+// generation word read before and written after the count: 3.4 us a barrier
+// of 32 CTAs instead of 1.7).  Returns false (in every thread of the CTA)
+// when the wait gave up; the status word then holds PK_ERR_TIMEOUT.  A
+// withheld CTA returns false without arriving.
+__device__ bool grid_sync(EvictHeader *h, uint32_t k, int32_t *status, const BarrierBound &bb) {
     __shared__ int ok;
     __syncthreads();
-    if (threadIdx.x == 0 && blockIdx.x == bb.withheld_cta) ok = 0;
-    if (threadIdx.x == 0 && blockIdx.x != bb.withheld_cta) {
-        ok = 1;
-        const unsigned int g = ld_acquire(&h->gen);
-        __threadfence();
-        if (atomicAdd(&h->arrive, 1u) == gridDim.x - 1) {
-            atomicExch(&h->arrive, 0u);
+    if (threadIdx.x == 0) {
+        ok = blockIdx.x != bb.withheld_cta;
+        if (ok) {
             __threadfence();
-            atomicAdd(&h->gen, 1u);
-        } else {
+            atomicAdd(&h->arrive, 1u);
+            const unsigned int all = (k + 1) * gridDim.x;
             uint32_t it = 0;
-            while (ld_acquire(&h->gen) == g) {
+            while (ld_acquire(&h->arrive) < all) {
                 if (++it > bb.spin_limit) {
                     ok = 0;
                     pk::set_status(status, PK_ERR_TIMEOUT);
                     break;
                 }
-                __nanosleep(100);
+                __nanosleep(20);
             }
+            __threadfence();
         }
-        __threadfence();
     }
     __syncthreads();
     return ok != 0;
 }
 
 constexpr uint32_t kPer = 4;  // elements per thread per iteration of the strided loops (loads in flight)
+constexpr uint32_t kWarps = kEvThreads / 32;
+constexpr uint32_t kSlotBuf = 512;  // slots of evicted entries that a warp collects before it writes them out
 
-// Block-collective append: thread t contributes c elements; returns the list
-// position of its first one, with one atomic on `counter` per CTA.  Every
-// thread of the CTA calls it.
-__device__ __forceinline__ unsigned long long block_append(uint32_t c, unsigned long long *counter) {
-    __shared__ uint32_t sh_warp[kEvThreads / 32];
-    __shared__ unsigned long long sh_base;
-    const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t incl = c;
+// The bucket of a 256-bin histogram (in global memory, complete) that holds ascending `rank`, by warp 0;
+// every thread of the CTA calls it.  sel[0]: the bucket, sel[1]: the rank within it, sel[2]: its count.
+__device__ __forceinline__ void pick_bucket(const unsigned int *hist, bool descending, unsigned long long rank,
+                                            unsigned long long *sel) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {  // 8 buckets per lane, then a warp scan
+        unsigned long long c[8], sum = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += y;
-    }
-    if (lane == 31) sh_warp[w] = incl;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t total = 0;
-        for (uint32_t u = 0; u < kEvThreads / 32; ++u) {
-            const uint32_t x = sh_warp[u];
-            sh_warp[u] = total;  // exclusive prefix over warps
-            total += x;
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t b = lane * 8 + u;
+            c[u] = __ldcg(hist + (descending ? 255 - b : b));
+            sum += c[u];
         }
-        sh_base = total ? atomicAdd(counter, (unsigned long long)total) : 0ull;
+        unsigned long long incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        unsigned long long excl = incl - sum;
+        if (rank >= excl && rank < incl) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (rank >= excl && rank < excl + c[u]) {
+                    const uint32_t b = lane * 8 + u;
+                    sel[0] = descending ? 255 - b : b;
+                    sel[1] = rank - excl;
+                    sel[2] = c[u];
+                }
+                excl += c[u];
+            }
+        }
     }
     __syncthreads();
-    return sh_base + sh_warp[w] + (incl - c);
+}
+
+// Shared-memory histogram increment of `bin` (256: none), one atomic per distinct bin of the warp.
+__device__ __forceinline__ void count_bin(unsigned int *sh_hist, uint32_t bin) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, bin);
+    if (bin < 256 && (peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0) atomicAdd(&sh_hist[bin], __popc(peers));
 }
 
 __device__ __forceinline__ bool bit(const uint32_t *bm, uint64_t i) { return (__ldcg(bm + (i >> 5)) >> (i & 31)) & 1u; }
-
-// Bulk prefetch of [p, p + bytes) into L2 (bytes a multiple of 16, p 16-byte aligned).
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
 
 // Length of the run of occupied positions (bitmap) starting at s, wrapping
 // around the table; at most `capacity`.
@@ -290,22 +316,23 @@ __device__ __noinline__ void compact_planned(pk_entry *table, unsigned long long
     }
 }
 
-__global__ void __launch_bounds__(kEvThreads, 1)
+__global__ void __launch_bounds__(kEvThreads, kEvBlocks)
 k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned long long *counter, uint64_t budget,
-        uint64_t keep, EvictHeader *h, uint32_t *bitmap, uint32_t *evbm, uint8_t *dist, unsigned long long *list,
-        uint32_t *list_slot, uint32_t *evicted, uint64_t evicted_cap, unsigned long long *n_evicted_out,
-        int32_t *status, BarrierBound bb) {
+        uint64_t keep, unsigned long long epoch, EvictHeader *h, uint32_t *bitmap, uint32_t *evbm, uint8_t *dist,
+        uint32_t *evicted, uint64_t evicted_cap, unsigned long long *n_evicted_out, int32_t *status, BarrierBound bb) {
     __shared__ unsigned int sh_hist[256];
-    __shared__ unsigned long long sh_sel[2];
-    __shared__ unsigned long long sh_removed;
+    __shared__ unsigned long long sh_sel[3];
+    __shared__ unsigned long long sh_count[2];
+    __shared__ unsigned long long sh_base;
+    __shared__ uint32_t sh_at[kWarps + 1];
+    __shared__ uint32_t sh_slots[kWarps][kSlotBuf];
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + tid;
     const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t mask = capacity - 1;
     const uint32_t kFull = 0xffffffffu;
-    // CTA-uniform strided loops: iteration `it` covers [it0 + it * span, +kPer*kEvThreads), element
-    // u of thread t at offset u*kEvThreads + t (coalesced per u)
-    const uint64_t span = nthreads * kPer, it0 = (uint64_t)blockIdx.x * kEvThreads * kPer;
+    // grid-uniform strided loops: an iteration covers kPer positions per thread, one per pass of the grid
+    const uint64_t span = nthreads * kPer;
 
     // 1. within the budget: nothing to do
     const unsigned long long count = __ldcg(counter);
@@ -313,41 +340,30 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
         if (gtid == 0 && n_evicted_out) *n_evicted_out = 0;
         return;
     }
-    if (tid == 0) sh_removed = 0;
+    const bool by_age = epoch >> 32 == 0;  // (a stamp holds 32 bits of its call's number)
+    if (tid < 256) sh_hist[tid] = 0;
+    if (tid < 2) sh_count[tid] = 0;
+    __syncthreads();
 
-    // 2. gather: occupancy bitmap, stamps and slots of occupied entries, stamp range
+    // 2. gather: occupancy bitmap, distances, counts, stamp range, age histogram
     unsigned long long lo = ~0ull, hi = 0;
-    if (tid == 0 && it0 < capacity) {
-        const uint64_t m = min((uint64_t)kPer * kEvThreads, capacity - it0);
-        prefetch_l2(&table[it0], (uint32_t)(m * sizeof(pk_entry)));
-        prefetch_l2(stamps + it0, (uint32_t)(m * 8));
-    }
-    for (uint64_t base = it0; base < capacity; base += span) {
-        if (tid == 0 && base + span < capacity) {  // the next iteration's entries and stamps
-            const uint64_t m = min((uint64_t)kPer * kEvThreads, capacity - base - span);
-            prefetch_l2(&table[base + span], (uint32_t)(m * sizeof(pk_entry)));
-            prefetch_l2(stamps + base + span, (uint32_t)(m * 8));
-        }
+    uint32_t max_index = 0, stamped = 0, unstamped = 0;
+    for (uint64_t base = 0; base < capacity; base += span) {
         uint4 k[kPer];
-        uint32_t sl[kPer];
         unsigned long long st[kPer];
 #pragma unroll
         for (uint32_t u = 0; u < kPer; ++u) {  // every load of the iteration at once (empty entries: stamp 0)
-            const uint64_t i = base + u * kEvThreads + tid;
+            const uint64_t i = base + u * nthreads + gtid;
             k[u] = make_uint4(0, 0, 0, 0);
-            sl[u] = 0;
             st[u] = 0;
             if (i < capacity) {
-                const uint4 *ep = reinterpret_cast<const uint4 *>(&table[i]);
-                k[u] = __ldcg(ep);
-                sl[u] = __ldcg(&table[i].slot);
+                k[u] = __ldcg(reinterpret_cast<const uint4 *>(&table[i]));
                 st[u] = __ldcg(stamps + i);
             }
         }
-        uint32_t c = 0;
 #pragma unroll
         for (uint32_t u = 0; u < kPer; ++u) {
-            const uint64_t i = base + u * kEvThreads + tid;
+            const uint64_t i = base + u * nthreads + gtid;
             const bool occ = !is_zero(k[u]);
             const uint32_t word = __ballot_sync(kFull, occ);
             if (lane == 0 && i < capacity) bitmap[i >> 5] = word;
@@ -355,18 +371,18 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
                 const uint64_t d = (i - ((((uint64_t)k[u].y << 32) | k[u].x) & mask)) & mask;
                 dist[i] = occ ? (uint8_t)(d < 255 ? d : 255) : (uint8_t)0;
             }
-            c += occ;
-        }
-        unsigned long long j = block_append(c, &h->n);
-#pragma unroll
-        for (uint32_t u = 0; u < kPer; ++u) {
-            if (!is_zero(k[u])) {
-                list[j] = st[u];
-                list_slot[j] = sl[u];
-                ++j;
+            uint32_t bin = 256;
+            if (occ && st[u]) {
+                const unsigned long long age = epoch - (st[u] >> 32);
+                bin = by_age && age < 255 ? (uint32_t)age : 255u;
+                ++stamped;
                 lo = st[u] < lo ? st[u] : lo;
                 hi = st[u] > hi ? st[u] : hi;
+                max_index = (uint32_t)st[u] > max_index ? (uint32_t)st[u] : max_index;
+            } else if (occ) {
+                ++unstamped;
             }
+            count_bin(sh_hist, bin);
         }
     }
 #pragma unroll
@@ -375,134 +391,148 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
         lo = l2 < lo ? l2 : lo;
         hi = h2 > hi ? h2 : hi;
     }
-    if (lane == 0 && hi >= lo) {
-        atomicMax(&h->inv_min, ~lo);
-        atomicMax(&h->max, hi);
+    max_index = __reduce_max_sync(kFull, max_index);
+    stamped = __reduce_add_sync(kFull, stamped);
+    unstamped = __reduce_add_sync(kFull, unstamped);
+    if (lane == 0) {
+        if (stamped) {
+            atomicMax(&h->inv_min, ~lo);
+            atomicMax(&h->max, hi);
+            atomicMax(&h->max_index, max_index);
+            atomicAdd_block(&sh_count[0], (unsigned long long)stamped);
+        }
+        if (unstamped) atomicAdd_block(&sh_count[1], (unsigned long long)unstamped);
     }
-    if (!grid_sync(h, status, bb)) return;
-    const unsigned long long n = __ldcg(&h->n);
-    unsigned long long prefix_v = 0;  // v, once selected
+    __syncthreads();
+    if (tid < 256 && sh_hist[tid]) atomicAdd(&h->age[tid], sh_hist[tid]);
+    if (tid == 0 && sh_count[0]) atomicAdd(&h->n_stamped, sh_count[0]);
+    if (tid == 0 && sh_count[1]) atomicAdd(&h->n_unstamped, sh_count[1]);
+    uint32_t barrier = 0;
+    if (!grid_sync(h, barrier++, status, bb)) return;
+    if (tid == 0) sh_count[0] = 0;  // from here: entries this CTA has removed
+    __syncthreads();
 
+    const unsigned long long n0 = __ldcg(&h->n_unstamped), n = n0 + __ldcg(&h->n_stamped);
+    unsigned long long v = 0;  // every stamp <= v goes (0: the entries without a stamp, as one group)
     if (n > keep) {
-        // 3. v = the stamp of ascending rank n - keep - 1
-        const unsigned long long smin = ~__ldcg(&h->inv_min), smax = __ldcg(&h->max);
-        const unsigned long long diff = smin ^ smax;
-        const int top = diff ? (63 - __clzll((long long)diff)) / 8 : -1;  // highest differing byte
-        unsigned long long prefix = top == 7 ? 0ull : top < 0 ? smin : smin >> (8 * (top + 1));
-        unsigned long long rank = n - keep - 1;
-        for (int byte = top, p = 0; byte >= 0; --byte, ++p) {
-            const int shift = 8 * byte;
-            for (uint32_t b = tid; b < 256; b += blockDim.x) sh_hist[b] = 0;
+        // 3. v, from the ascending rank n - keep - 1 of the last stamp to go
+        if (n - keep > n0) {
+            const unsigned long long smin = ~__ldcg(&h->inv_min), smax = __ldcg(&h->max);
+            pick_bucket(h->age, true, n - keep - 1 - n0, sh_sel);  // oldest first
+            const unsigned long long age = sh_sel[0];
+            unsigned long long rank = sh_sel[1], left = sh_sel[2];
+            // the candidates' range [clo, chi]
+            unsigned long long clo = age < 255 ? (epoch - age) << 32 : 0ull;
+            unsigned long long chi = age < 255 ? clo | __ldcg(&h->max_index) : by_age ? ((epoch - 254) << 32) - 1 : ~0ull;
+            clo = clo > smin ? clo : smin;
+            chi = chi < smax ? chi : smax;
             __syncthreads();
-            for (uint64_t base = it0; base < n; base += span) {
-                unsigned long long x[kPer];
+            for (uint32_t p = 0; rank + 1 < left && clo < chi; ++p) {  // the bucket goes only in part: split it
+                const int bits = 64 - __clzll((long long)(chi - clo));
+                const int shift = bits > 8 ? bits - 8 : 0;
+                unsigned int *hist = h->hist[p % kPasses];
+                if (tid < 256) sh_hist[tid] = 0;
+                __syncthreads();
+                for (uint64_t base = 0; base < capacity; base += span) {
+                    unsigned long long x[kPer];
 #pragma unroll
-                for (uint32_t u = 0; u < kPer; ++u) {
-                    const uint64_t j = base + u * kEvThreads + tid;
-                    x[u] = j < n ? __ldcg(list + j) : 0ull;
-                }
-#pragma unroll
-                for (uint32_t u = 0; u < kPer; ++u) {
-                    const uint64_t j = base + u * kEvThreads + tid;
-                    const bool cand = j < n && (byte == top || (x[u] >> (shift + 8)) == prefix);
-                    const uint32_t bin = cand ? (uint32_t)(x[u] >> shift) & 255u : 256u;
-                    const uint32_t peers = __match_any_sync(kFull, bin);
-                    if (bin < 256 && (peers & ((1u << lane) - 1u)) == 0) atomicAdd(&sh_hist[bin], __popc(peers));
-                }
-            }
-            __syncthreads();
-            for (uint32_t b = tid; b < 256; b += blockDim.x)
-                if (sh_hist[b]) atomicAdd(&h->hist[p][b], sh_hist[b]);
-            if (!grid_sync(h, status, bb)) return;
-            if (tid < 32) {  // bucket holding `rank`: 8 buckets per lane, then a warp scan
-                unsigned long long c[8], sum = 0;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    c[u] = __ldcg(&h->hist[p][lane * 8 + u]);
-                    sum += c[u];
-                }
-                unsigned long long incl = sum;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long y = __shfl_up_sync(kFull, incl, o);
-                    if (lane >= (uint32_t)o) incl += y;
-                }
-                unsigned long long excl = incl - sum;
-                if (rank >= excl && rank < incl) {
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        if (rank >= excl && rank < excl + c[u]) {
-                            sh_sel[0] = lane * 8 + u;
-                            sh_sel[1] = rank - excl;
-                        }
-                        excl += c[u];
+                    for (uint32_t u = 0; u < kPer; ++u) {
+                        const uint64_t i = base + u * nthreads + gtid;
+                        x[u] = i < capacity ? __ldcg(stamps + i) : 0ull;
                     }
+#pragma unroll
+                    for (uint32_t u = 0; u < kPer; ++u)  // (stamps of the candidates are not zero: clo >= smin)
+                        count_bin(sh_hist, x[u] >= clo && x[u] <= chi ? (uint32_t)((x[u] - clo) >> shift) : 256u);
                 }
+                __syncthreads();
+                if (tid < 256 && sh_hist[tid]) atomicAdd(&hist[tid], sh_hist[tid]);
+                if (!grid_sync(h, barrier++, status, bb)) return;
+                pick_bucket(hist, false, rank, sh_sel);
+                clo += sh_sel[0] << shift;
+                const unsigned long long top = clo + ((1ull << shift) - 1);
+                chi = top < chi ? top : chi;
+                rank = sh_sel[1];
+                left = sh_sel[2];
+                // a row is used again kPasses passes later: cleared two barriers before that, when every CTA has read it
+                if (p + 2 >= kPasses && blockIdx.x == 0 && tid < 256) h->hist[(p + 2) % kPasses][tid] = 0;
+                __syncthreads();
             }
-            __syncthreads();
-            prefix = (prefix << 8) | sh_sel[0];
-            rank = sh_sel[1];
-            __syncthreads();
+            v = chi;
         }
-        const unsigned long long v = prefix;
-        prefix_v = v;
 
-        // 4a. the slots of the removed entries, one atomic per CTA and iteration
+        // 4a. the evicted positions as a bitmap, and their slots, collected per warp in shared memory
+        const uint32_t warp = tid >> 5;
         unsigned long long removed = 0;
-        for (uint64_t base = it0; base < n; base += span) {
-            bool ev[kPer];
-            uint32_t c = 0;
-#pragma unroll
-            for (uint32_t u = 0; u < kPer; ++u) {
-                const uint64_t j = base + u * kEvThreads + tid;
-                ev[u] = j < n && __ldcg(list + j) <= v;
-                c += ev[u];
+        uint32_t have = 0;  // slots in this warp's buffer
+        auto put = [&](unsigned long long first) {  // the warp's buffer to evicted[first ..)
+            __syncwarp();
+            for (uint32_t j = lane; j < have; j += 32) {
+                if (first + j < evicted_cap) evicted[first + j] = sh_slots[warp][j];
+                else if (evicted) pk::set_status(status, PK_ERR_ARG);
             }
-            unsigned long long o = block_append(c, &h->n_evicted);
-            removed += c;
-#pragma unroll
-            for (uint32_t u = 0; u < kPer; ++u) {
-                if (ev[u]) {
-                    const uint64_t j = base + u * kEvThreads + tid;
-                    if (o < evicted_cap) evicted[o] = __ldcg(list_slot + j);
-                    else if (evicted) pk::set_status(status, PK_ERR_ARG);
-                    ++o;
-                }
-            }
-        }
-        if (removed) atomicAdd_block(&sh_removed, removed);
-        __syncthreads();
-        if (tid == 0 && sh_removed) atomicAdd(counter, (unsigned long long)(-(long long)sh_removed));
-
-        // 4b. the evicted positions as a bitmap
-        for (uint64_t base = it0; base < capacity; base += span) {
+            __syncwarp();
+        };
+        for (uint64_t base = 0; base < capacity; base += span) {
             unsigned long long st[kPer];
-            uint32_t wd[kPer];
+            uint32_t wd[kPer], sl[kPer];
+            bool ev[kPer];
 #pragma unroll
             for (uint32_t u = 0; u < kPer; ++u) {
-                const uint64_t i = base + u * kEvThreads + tid;
-                st[u] = i < capacity ? __ldcg(stamps + i) : 0ull;
+                const uint64_t i = base + u * nthreads + gtid;
+                st[u] = i < capacity ? __ldcg(stamps + i) : ~0ull;
                 wd[u] = i < capacity ? __ldcg(bitmap + (i >> 5)) : 0u;
             }
 #pragma unroll
             for (uint32_t u = 0; u < kPer; ++u) {
-                const uint64_t i = base + u * kEvThreads + tid;
-                const bool ev = ((wd[u] >> lane) & 1u) && st[u] <= v;
-                const uint32_t word = __ballot_sync(kFull, ev);
+                const uint64_t i = base + u * nthreads + gtid;
+                ev[u] = ((wd[u] >> lane) & 1u) && st[u] <= v;
+                sl[u] = ev[u] ? __ldcg(&table[i].slot) : 0u;
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < kPer; ++u) {
+                const uint64_t i = base + u * nthreads + gtid;
+                const uint32_t word = __ballot_sync(kFull, ev[u]);
                 if (lane == 0 && i < capacity) evbm[i >> 5] = word;
+                if (ev[u]) sh_slots[warp][have + __popc(word & ((1u << lane) - 1u))] = sl[u];
+                have += __popc(word);
+            }
+            if (have + 32 * kPer > kSlotBuf) {  // the next iteration may not fit
+                unsigned long long first = 0;
+                if (lane == 0) first = atomicAdd(&h->n_evicted, (unsigned long long)have);
+                put(__shfl_sync(kFull, first, 0));
+                removed += have;
+                have = 0;
             }
         }
+        // what is left in the buffers: one atomic per CTA
+        if (lane == 0) sh_at[warp] = have;
+        if (lane == 0 && removed) atomicAdd_block(&sh_count[0], removed);
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t total = 0;
+            for (uint32_t u = 0; u < kWarps; ++u) {
+                const uint32_t x = sh_at[u];
+                sh_at[u] = total;
+                total += x;
+            }
+            sh_base = total ? atomicAdd(&h->n_evicted, (unsigned long long)total) : 0ull;
+            const unsigned long long gone = sh_count[0] + total;
+            if (gone) atomicAdd(counter, (unsigned long long)(-(long long)gone));
+        }
+        __syncthreads();
+        put(sh_base + sh_at[warp]);
     }
-    if (!grid_sync(h, status, bb)) return;
+    if (!grid_sync(h, barrier++, status, bb)) return;
+    if (gtid == 0 && n_evicted_out) *n_evicted_out = __ldcg(&h->n_evicted);
     if (n > keep) {
-        // 4c. compaction: one thread per bitmap word, for the clusters that start in it.  Clusters
+        // 4b. compaction: one thread per bitmap word, for the clusters that start in it and lose an entry.  Clusters
         // that end within the 64 positions of the word and the next one are planned in registers
         // from the occupancy, evicted and distance bytes; the word's moves then go out four loads
         // at a time.  Longer clusters take compact_planned (the same plan, 32 positions at a time),
         // tables below 64 entries and clusters beyond kPlanMax compact_walk.
-        const unsigned long long v = prefix_v;
         const uint64_t n_words = (capacity + 31) / 32;
-        for (uint64_t w = gtid; w < n_words; w += nthreads) {
+        // 32 words per warp, the warps in turn over the CTAs (a small table's words spread over the SMs)
+        for (uint64_t w = ((uint64_t)(tid >> 5) * gridDim.x + blockIdx.x) * 32 + lane; w < n_words; w += nthreads) {
             const uint32_t occ_lo = __ldcg(bitmap + w);
             if (!occ_lo) continue;
             const uint32_t before = bit(bitmap, (w * 32 + mask) & mask);  // the position before bit 0
@@ -518,6 +548,7 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
             const uint64_t w1 = (w + 1) % n_words;  // the next word (wrapping)
             const uint64_t occ = occ_lo | ((uint64_t)__ldcg(bitmap + w1) << 32);
             const uint64_t evw = __ldcg(evbm + w) | ((uint64_t)__ldcg(evbm + w1) << 32);
+            if (!evw && (~occ >> 32)) continue;  // nothing goes in the window, and no cluster of it leaves the window
             uint32_t dv[16];
             {
                 const uint4 *d0 = reinterpret_cast<const uint4 *>(dist + w * 32);
@@ -536,6 +567,7 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
                 const uint64_t rest = ~(occ >> b);
                 const uint32_t run = rest ? __ffsll((long long)rest) - 1 : 64 - b;
                 if (b + run < 64) {  // the cluster ends inside the window
+                    if (!((evw >> b) & ((1ull << run) - 1ull))) continue;  // and keeps every entry
                     uint64_t taken = 0;  // relative to b
                     for (uint32_t j = 0; j < run; ++j) {
                         const uint32_t p = b + j;
@@ -600,12 +632,11 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
             }
         }
     }
-    if (!grid_sync(h, status, bb)) return;
-    if (gtid == 0 && n_evicted_out) *n_evicted_out = __ldcg(&h->n_evicted);
 }
 
 }  // namespace
 
+// (12 bytes per entry, once a list of stamps and slots, are not used: the size that callers allocate by is kept)
 uint64_t pk_evict_scratch_bytes_impl(uint64_t capacity) {
     return kHeaderBytes + 2 * bitmap_bytes(capacity) + 8 * capacity + 4 * capacity + ((capacity + 255) & ~255ull);
 }
@@ -636,8 +667,8 @@ cudaError_t pk_launch_evict(const pk_ctx *ctx, uint64_t budget, uint64_t keep, v
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = evict_resident(dev, &resident);
     if (e != cudaSuccess) return e;
-    // every CTA resident (the barriers need it); no more CTAs than the table has rows of kEvThreads entries
-    const uint64_t want = (ctx->capacity + kEvThreads - 1) / kEvThreads;
+    // every CTA resident (the barriers need it); no more CTAs than the table has rows of kEvRows entries
+    const uint64_t want = (ctx->capacity + kEvRows - 1) / kEvRows;
     const unsigned grid = (unsigned)(want < resident ? want : resident);
     uint8_t *base = static_cast<uint8_t *>(scratch);
     EvictHeader *h = reinterpret_cast<EvictHeader *>(base);
@@ -645,9 +676,6 @@ cudaError_t pk_launch_evict(const pk_ctx *ctx, uint64_t budget, uint64_t keep, v
     const uint64_t bmb = bitmap_bytes(ctx->capacity);
     uint32_t *evbm = reinterpret_cast<uint32_t *>(base + kHeaderBytes + bmb);
     uint8_t *dist = base + kHeaderBytes + 2 * bmb;
-    unsigned long long *list =
-        reinterpret_cast<unsigned long long *>(dist + ((ctx->capacity + 255) & ~255ull));
-    uint32_t *list_slot = reinterpret_cast<uint32_t *>(list + ctx->capacity);
     e = cudaMemsetAsync(h, 0, sizeof(EvictHeader), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -661,7 +689,7 @@ cudaError_t pk_launch_evict(const pk_ctx *ctx, uint64_t budget, uint64_t keep, v
     cfg.numAttrs = 1;
     const BarrierBound bb{spin_limit == 0 || spin_limit > kSpinLimit ? kSpinLimit : spin_limit,
                           withhold_first_cta ? 0u : 0xffffffffu};
-    e = cudaLaunchKernelEx(&cfg, k_evict, ctx->table, ctx->stamps, ctx->capacity, ctx->counter_dev, budget, keep, h,
-                           bitmap, evbm, dist, list, list_slot, evicted, evicted_cap, n_evicted, status, bb);
+    e = cudaLaunchKernelEx(&cfg, k_evict, ctx->table, ctx->stamps, ctx->capacity, ctx->counter_dev, budget, keep,
+                           ctx->epoch, h, bitmap, evbm, dist, evicted, evicted_cap, n_evicted, status, bb);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
