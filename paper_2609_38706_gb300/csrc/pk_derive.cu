@@ -17,6 +17,7 @@
 
 #include "pk_device.cuh"
 #include "pk_internal.h"
+#include "pk_pair.cuh"
 #include "pk_sha256.cuh"
 
 namespace {
@@ -27,15 +28,25 @@ using pk::set_status;
 // Descriptor digests: one warp per descriptor.  The warp copies the encoding
 // into shared memory with coalesced byte loads (32 bytes per round trip), then
 // one lane hashes it.  Encodings longer than the staging area are hashed from
-// global memory.
+// global memory.  Two forms:
+//   hash_descriptor        pads the encoding in shared memory and hashes its
+//                          words with the 16-round code: where the descriptors
+//                          set the time, in small batches (key derivation of
+//                          512 chunks of 16 tokens under 16 descriptors of about
+//                          200 bytes 26.1 -> 24.8 us);
+//   hash_descriptor_bytes  takes it byte by byte, in straight-line rounds: in the
+//                          launch of a large batch, whose chunk digests hide it
+//                          and compile to slower code beside a third copy of the
+//                          16-round code (small-block key derivation 613.8 against
+//                          616.1 us).
 // ---------------------------------------------------------------------------
 constexpr int kDescWarps = 4;
 constexpr int kDescStage = 2048;
 
-// Warp `warp` of the calling block hashes descriptor j (all 32 lanes call).
-__device__ __forceinline__ void hash_descriptor(uint8_t *stage, const uint8_t *enc, uint64_t enc_bytes,
-                                                const int64_t *enc_off, uint32_t j,
-                                                uint8_t *digests, int32_t *status) {
+// The calling warp hashes descriptor j (all 32 lanes call).
+__device__ __forceinline__ void hash_descriptor_bytes(uint8_t *stage, const uint8_t *enc, uint64_t enc_bytes,
+                                                      const int64_t *enc_off, uint32_t j,
+                                                      uint8_t *digests, int32_t *status) {
     const uint32_t lane = threadIdx.x & 31;
     const int64_t a = __ldcg(enc_off + j), b = __ldcg(enc_off + j + 1);
     if (a < 0 || b < a || (uint64_t)b > enc_bytes) {
@@ -52,15 +63,58 @@ __device__ __forceinline__ void hash_descriptor(uint8_t *stage, const uint8_t *e
     if (lane == 0) pk::sha256_bytes(staged ? stage : enc + a, (uint64_t)len, digests + 32ull * j);
 }
 
+// stage: kDescStage bytes, 16-byte aligned; sK: the round constants.
+__device__ __forceinline__ void hash_descriptor(uint8_t *stage, const uint32_t *sK, const uint8_t *enc, uint64_t enc_bytes,
+                                                const int64_t *enc_off, uint32_t j,
+                                                uint8_t *digests, int32_t *status) {
+    const uint32_t lane = threadIdx.x & 31;
+    const int64_t a = __ldcg(enc_off + j), b = __ldcg(enc_off + j + 1);
+    if (a < 0 || b < a || (uint64_t)b > enc_bytes) {
+        if (lane == 0) set_status(status, PK_ERR_ARG);
+        return;
+    }
+    const int64_t len = b - a, blocks = (len + 8) / 64 + 1;
+    if (64 * blocks > kDescStage) {
+        if (lane == 0) pk::sha256_bytes(enc + a, (uint64_t)len, digests + 32ull * j);
+        return;
+    }
+    uint32_t *words = reinterpret_cast<uint32_t *>(stage);
+    for (int64_t i = (len >> 2) + lane; i < 16 * blocks; i += 32) words[i] = 0u;
+    __syncwarp();
+#pragma unroll 4
+    for (int64_t i = lane; i < len; i += 32) stage[i] = __ldcg(enc + a + i);
+    if (lane == 0) {
+        stage[len] = 0x80u;
+        words[16 * blocks - 1] = pk::bswap32((uint32_t)len * 8u);  // (len < 2^11)
+    }
+    __syncwarp();
+    if (lane == 0) {
+        uint32_t st[8], w[16];
+        pk::init_state(st);
+#pragma unroll 1
+        for (int64_t blk = 0; blk < blocks; ++blk) {
+#pragma unroll
+            for (int t = 0; t < 16; ++t) w[t] = pk::bswap32(words[16 * blk + t]);
+            pk::compress_rolled(st, w, sK);
+        }
+        uint4 *q = reinterpret_cast<uint4 *>(digests + 32ull * j);
+        q[0] = make_uint4(pk::bswap32(st[0]), pk::bswap32(st[1]), pk::bswap32(st[2]), pk::bswap32(st[3]));
+        q[1] = make_uint4(pk::bswap32(st[4]), pk::bswap32(st[5]), pk::bswap32(st[6]), pk::bswap32(st[7]));
+    }
+}
+
 __global__ void __launch_bounds__(32 * kDescWarps)
 k_digest_descriptors(const uint8_t *enc, uint64_t enc_bytes, const int64_t *enc_off,
                      uint32_t D, uint8_t *digests, int32_t *status) {
     __shared__ __align__(16) uint8_t stage[kDescWarps][kDescStage];
+    __shared__ uint32_t sK[64];
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) sK[i] = pk::kSha256K[i];
+    __syncthreads();
     pk::pdl_launch_dependents();
     pk::pdl_wait(enc, enc_off, digests, status);
     const uint32_t warp = threadIdx.x >> 5;
     const uint32_t j = blockIdx.x * kDescWarps + warp;
-    if (j < D) hash_descriptor(stage[warp], enc, enc_bytes, enc_off, j, digests, status);
+    if (j < D) hash_descriptor(stage[warp], sK, enc, enc_bytes, enc_off, j, digests, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -349,7 +403,7 @@ k_chunk_digest(const int32_t *tokens, const int64_t *tok_off,
         const uint32_t warp = threadIdx.x >> 5;
         const uint32_t j = blockIdx.x * (kDigestBlock / 32) + warp;
         uint8_t *stage = reinterpret_cast<uint8_t *>(ring[0]) + warp * kDescStage;  // 4 x 2 KiB of the ring
-        if (j < dw.D) hash_descriptor(stage, enc, dw.enc_bytes, enc_off, j, digests, dstatus);
+        if (j < dw.D) hash_descriptor_bytes(stage, enc, dw.enc_bytes, enc_off, j, digests, dstatus);
         pk::pdl_launch_dependents();
         return;
     }
@@ -370,6 +424,81 @@ k_chunk_digest(const int32_t *tokens, const int64_t *tok_off,
         __syncwarp();
     }
     pk::pdl_launch_dependents();
+}
+
+// The chunk digests of a batch of few chunks, by pairs of warps (pk_pair.cuh): 16 chunks per pair.  CTA c of the
+// work CTAs serves pairs [c * P / ctas, (c + 1) * P / ctas), at most three.
+struct ChunkWords {
+    const int32_t *src;  // the chunk's tokens (nullptr: a lane without a chunk)
+    uint32_t C;
+    uint32_t last;  // the block that holds the length
+    __device__ __forceinline__ bool inside(uint32_t b) const { return src && 16 * b + 16 <= C; }
+    __device__ __forceinline__ const uint32_t *block(uint32_t b) const {
+        return reinterpret_cast<const uint32_t *>(src) + 16 * b;
+    }
+    __device__ __forceinline__ uint32_t load(uint32_t b, uint32_t t) const {
+        const uint32_t i = 16 * b + t;
+        return src && i < C ? (uint32_t)__ldcg(src + i) : 0u;
+    }
+    __device__ __forceinline__ int tail(uint32_t) const { return -1; }
+    __device__ __forceinline__ uint32_t tail_word(uint32_t) const { return 0u; }
+    __device__ __forceinline__ uint32_t word(uint32_t b, uint32_t t, uint32_t x) const {
+        const uint32_t i = 16 * b + t;
+        if (i < C) return pk::bswap32(x);
+        const uint64_t bits = (uint64_t)C * 32u;
+        if (b == last && t >= 14) return t == 14 ? (uint32_t)(bits >> 32) : (uint32_t)bits;
+        return i == C ? 0x80000000u : 0u;
+    }
+};
+
+__global__ void __launch_bounds__(pk::kPairThreads)
+k_chunk_digest_pairs(const int32_t *tokens, const int64_t *tok_off, const int64_t *key_off, uint32_t R, uint32_t C,
+                     const __grid_constant__ PadKW pad, uint8_t *keys, const __grid_constant__ DescWork dw, uint32_t one) {
+    extern __shared__ __align__(16) uint8_t pair_smem[];
+    pk::PairSmem &sm = *reinterpret_cast<pk::PairSmem *>(pair_smem);
+    static_assert(sizeof(sm.ring) >= (size_t)kDescStage * kDescWarps, "descriptor staging fits in the rings");
+    if (blockIdx.x < dw.desc_blocks) {
+        const uint8_t *enc = dw.enc;
+        const int64_t *enc_off = dw.enc_off;
+        uint8_t *digests = dw.digests;
+        int32_t *dstatus = dw.status;
+        uint32_t *sK = sm.zero;  // (not otherwise used by this CTA)
+        for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) sK[i] = pk::kSha256K[i];
+        __syncthreads();
+        pk::pdl_wait(enc, enc_off, digests, dstatus);
+        const uint32_t warp = threadIdx.x >> 5;
+        const uint32_t j = blockIdx.x * kDescWarps + warp;
+        uint8_t *stage = reinterpret_cast<uint8_t *>(sm.ring) + warp * kDescStage;
+        if (warp < kDescWarps && j < dw.D) hash_descriptor(stage, sK, enc, dw.enc_bytes, enc_off, j, digests, dstatus);
+        pk::pdl_launch_dependents();
+        return;
+    }
+    pair_tables(sm, pad.kw);
+    __syncthreads();
+    pk::pdl_wait(tokens, tok_off, key_off, keys);
+    const int64_t total = __ldcg(key_off + R);
+    const int64_t P = (total + pk::kPairMsgs - 1) / pk::kPairMsgs;
+    const int64_t ctas = gridDim.x - dw.desc_blocks, c = blockIdx.x - dw.desc_blocks;
+    const pk::PairRole role = pk::pair_role();
+    const int64_t p = c * P / ctas + role.pair;
+    if (role.pair < pk::kPairs && p < (c + 1) * P / ctas) {
+        const pk::SplitLane l = pk::split_lane(one);
+        const int64_t g0 = p * pk::kPairMsgs, g = g0 + ((threadIdx.x & 31) >> 1);
+        const bool pad_block = C % 16 == 0;
+        const uint32_t blocks = pad_block ? C / 16 : (C * 4ull + 9 + 63) / 64;
+        if (role.sched) {
+            const uint32_t r = pk::lane_request_guess(key_off, R, g0, total, g);
+            const int32_t *src = nullptr;
+            if (g < total) src = tokens + __ldcg(tok_off + r) + (g - __ldcg(key_off + r)) * (int64_t)C;
+            pair_schedule(sm, role.pair, l, blocks, ChunkWords{src, C, pad_block ? blocks : blocks - 1});
+        } else {
+            uint32_t st[4];
+            pair_rounds(sm, role.pair, l, blocks, pad_block, st);
+            if (g < total) pair_store(keys + 32 * g, l, st);
+        }
+    }
+    pk::pdl_launch_dependents();
+    __syncthreads();  // stay resident until every pair's barriers are through
 }
 
 // ---------------------------------------------------------------------------
@@ -911,15 +1040,17 @@ k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *d
 
 unsigned grid_for(uint64_t n, unsigned block) { return (unsigned)((n + block - 1) / block); }
 
-// Shared memory of the four-pair chain CTA: its four ChainSmem (100 KiB), padded past half of an SM's
-// shared memory so that no SM holds two of these CTAs (the launch becomes resident while the chunk digests
-// drain, and would otherwise stack CTAs on the SMs that free up first).
-constexpr size_t kChainPackedSmem = 116 * 1024;
-constexpr size_t kChainHalfSmem = 76 * 1024;  // past a third: at most two CTAs per SM
-static_assert(kChainPackedSmem >= kChainPairs * sizeof(ChainSmem), "four pairs fit");
+// Dynamic shared memory of the kernels whose CTAs must not stack on an SM: padded past half of an SM's, or past a
+// third for two per SM (a launch that becomes resident while its predecessor drains otherwise stacks CTAs on the SMs
+// that free up first).
+constexpr size_t kOnePerSm = 116 * 1024;
+constexpr size_t kTwoPerSm = 76 * 1024;
+static_assert(kOnePerSm >= kChainPairs * sizeof(ChainSmem) && kOnePerSm >= 4 * sizeof(SplitSmem) &&
+                  kTwoPerSm >= sizeof(SplitSmem) && kOnePerSm >= sizeof(pk::PairSmem),
+              "the kernels' shared memory fits");
 
-// Raise the four-pair chain CTA's shared-memory limit once per device.
-cudaError_t chain_packed_attr() {
+// Raise those kernels' shared-memory limit, once per device.
+cudaError_t raise_smem_limits() {
     static std::mutex mu;
     static bool done[256] = {};
     int dev = 0;
@@ -927,35 +1058,17 @@ cudaError_t chain_packed_attr() {
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
-    if (!done[dev]) {
-        e = cudaFuncSetAttribute(k_chain<pk::kAddsPlain, pk::kAddsFma>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kChainPackedSmem);
-        if (e != cudaSuccess) return e;
-        done[dev] = true;
-    }
-    return cudaSuccess;
-}
-
-static_assert(kChainPackedSmem >= 4 * sizeof(SplitSmem), "four split pairs fit");
-// Raise the two-lane chain CTAs' shared-memory limit once per device.
-cudaError_t chain_split_attr() {
-    static std::mutex mu;
-    static bool done[256] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!done[dev]) {
-        e = cudaFuncSetAttribute(k_chain_split<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_chain_split<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_chain_split<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainPackedSmem);
-        if (e != cudaSuccess) return e;
-        done[dev] = true;
-    }
-    return cudaSuccess;
+    if (done[dev]) return cudaSuccess;
+    auto raise = [&](auto *kernel) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOnePerSm);
+    };
+    raise(k_chunk_digest_pairs);
+    raise(k_chain_split<1>);
+    raise(k_chain_split<3>);
+    raise(k_chain_split<4>);
+    raise(k_chain<pk::kAddsPlain, pk::kAddsFma>);
+    done[dev] = e == cudaSuccess;
+    return e;
 }
 
 }  // namespace
@@ -994,6 +1107,8 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     for (int t = 0; t < 64; ++t) pad.kw[t] = ctx->pad_kw[t];
     const bool chunks = R > 0 && key_capacity > 0;
     const uint32_t one = 1u;
+    if (chunks) e = raise_smem_limits();
+    if (e != cudaSuccess) return e;
     if (!chunks) {
         if (dw.desc_blocks)
             e = pk_launch(k_chunk_digest<pk::kAddsPlain>, dw.desc_blocks, kDigestBlock, s, tokens, tok_off,
@@ -1006,10 +1121,24 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     const uint64_t warps = (key_capacity + 31) / 32;
     const bool fma = ctx->sm_count > 0 && warps >= (uint64_t)kFmaWarps * 4u * ctx->sm_count;
     const unsigned grid = grid_for(key_capacity, kDigestBlock) + dw.desc_blocks;
-    e = fma ? pk_launch(k_chunk_digest<pk::kAddsFma>, grid, kDigestBlock, s, tokens, tok_off, (const int64_t *)key_off,
-                        R, C, pad, keys, dw, one)
-            : pk_launch(k_chunk_digest<pk::kAddsPlain>, grid, kDigestBlock, s, tokens, tok_off,
-                        (const int64_t *)key_off, R, C, pad, keys, dw, one);
+    // Few chunks: pairs of warps, at most three per SM, on the SMs that the descriptors and the offsets kernel, still
+    // running when this launch comes up, leave free.  Key derivation of N chunks (8 per request), one lane per chunk |
+    // pairs, in us: chunks of 256, N = 16: 38.0 | 31.4, 2400: 45.4 | 39.2, 7000: 45.6 | 44.6; chunks of 64: 21.1 |
+    // 20.9, 28.0 | 27.5, 28.3 | 28.9; chunks of 16: 19.7 | 17.5, 26.2 | 24.8, 26.7 | 25.3.
+    const uint32_t desc_sms = enc_off ? grid_for(D, kDescWarps) : 0;
+    const uint32_t work = ctx->sm_count > desc_sms + 1 ? ctx->sm_count - desc_sms - 1 : 0;
+    if (C <= 1u << 30 && key_capacity <= (uint64_t)pk::kPairMsgsPerSm * work) {
+        dw.desc_blocks = desc_sms;
+        const uint64_t pairs = (key_capacity + pk::kPairMsgs - 1) / pk::kPairMsgs;
+        e = pk_launch_smem(k_chunk_digest_pairs, (unsigned)(pairs < work ? pairs : work) + desc_sms, pk::kPairThreads,
+                           kOnePerSm, s, tokens, tok_off, (const int64_t *)key_off, R, C, pad, keys, dw, one);
+    } else if (fma) {
+        e = pk_launch(k_chunk_digest<pk::kAddsFma>, grid, kDigestBlock, s, tokens, tok_off, (const int64_t *)key_off, R, C,
+                      pad, keys, dw, one);
+    } else {
+        e = pk_launch(k_chunk_digest<pk::kAddsPlain>, grid, kDigestBlock, s, tokens, tok_off, (const int64_t *)key_off, R, C,
+                      pad, keys, dw, one);
+    }
     if (e != cudaSuccess) return e;
     // Chains, by pairs of 16 requests per SM (rounded up).  Key derivation of R prompts of 32 chunks of 16
     // tokens, measured, in us, for: two lanes per request, one pair per CTA | three | four | one lane per request:
@@ -1020,27 +1149,19 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     const uint32_t per_sm = sms ? grid_for(groups, sms) : 1;
     if (per_sm <= 2) {
         // Shared memory padded so that no SM takes more than its share of the CTAs (R = 4864 without: 123 us).
-        const size_t smem = per_sm == 1 ? kChainPackedSmem : kChainHalfSmem;
-        e = chain_split_attr();
-        if (e == cudaSuccess)
-            e = pk_launch_smem(k_chain_split<1>, groups, 64, smem, s, (const int64_t *)key_off, desc_idx,
+        const size_t smem = per_sm == 1 ? kOnePerSm : kTwoPerSm;
+        e = pk_launch_smem(k_chain_split<1>, groups, 64, smem, s, (const int64_t *)key_off, desc_idx,
                                (const uint8_t *)digests, R, D, keys, groups, one);
     } else if (per_sm == 3) {
-        e = chain_split_attr();
-        if (e == cudaSuccess)
-            e = pk_launch_smem(k_chain_split<3>, sms, 32 * split_warps(3), kChainPackedSmem, s, (const int64_t *)key_off,
+        e = pk_launch_smem(k_chain_split<3>, sms, 32 * split_warps(3), kOnePerSm, s, (const int64_t *)key_off,
                                desc_idx, (const uint8_t *)digests, R, D, keys, groups, one);
     } else if (per_sm == 4) {
-        e = chain_split_attr();
-        if (e == cudaSuccess)
-            e = pk_launch_smem(k_chain_split<4>, sms, 32 * split_warps(4), kChainPackedSmem, s, (const int64_t *)key_off, desc_idx,
+        e = pk_launch_smem(k_chain_split<4>, sms, 32 * split_warps(4), kOnePerSm, s, (const int64_t *)key_off, desc_idx,
                                (const uint8_t *)digests, R, D, keys, groups, one);
     } else {
         const uint32_t g32 = grid_for(R, kChainLanes);
-        e = chain_packed_attr();
         const uint32_t grid = g32 <= 4 * sms ? sms : grid_for(g32, 4);
-        if (e == cudaSuccess)
-            e = pk_launch_smem(k_chain<pk::kAddsPlain, pk::kAddsFma>, grid, 8 * kChainLanes, kChainPackedSmem, s,
+        e = pk_launch_smem(k_chain<pk::kAddsPlain, pk::kAddsFma>, grid, 8 * kChainLanes, kOnePerSm, s,
                                (const int64_t *)key_off, desc_idx, (const uint8_t *)digests, R, D, keys, g32, one);
     }
     if (e != cudaSuccess) return e;
