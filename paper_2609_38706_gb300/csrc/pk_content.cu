@@ -212,9 +212,10 @@ cudaError_t pk_launch_content_digests(const uint8_t *const *bytes, const uint64_
         const uint32_t m[16] = {0x80000000u, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, (uint32_t)(kTreeBlock * 8)};
         pk::kw_table(m, pad.kw);
     }
-    // Blocks of a level up to which pairs of warps serve it (a level of 16 to 1,238 blocks 26 -> 14 us), and from
-    // which the multiply-add round form is used (3 warps per SM sub-partition, as for the chunk digests).
-    const uint64_t sms = device_sms(), pairs_to = pk::kPairMsgsPerSm * sms, fma_from = 3ull * 4 * 32 * sms;
+    // Blocks of a level up to which pairs of warps serve it (a level of 16 to 1,238 blocks 26 -> 14 us), and above
+    // which two warps share a sub-partition, where the multiply-add round form is the faster one (the first level of
+    // 16 tensors of 40 MB, 1,238 warps: the call 132 -> 123 us; 1 GiB: 1395 -> 1213 us).
+    const uint64_t sms = device_sms(), pairs_to = pk::kPairMsgsPerSm * sms, fma_above = 32ull * 4 * sms;
     const uint32_t one = 1u;
     for (uint32_t j0 = 0; j0 < n; j0 += kMaxSeg) {
         const uint32_t cnt = n - j0 < kMaxSeg ? n - j0 : kMaxSeg;
@@ -246,7 +247,7 @@ cudaError_t pk_launch_content_digests(const uint8_t *const *bytes, const uint64_
             const cudaError_t e = threads <= pairs_to
                                       ? pk_launch(k_tree_level_pairs, (unsigned)(pairs < sms ? pairs : sms),
                                                   pk::kPairThreads, s, lv, pad, one)
-                                  : sms && threads >= fma_from
+                                  : sms && threads > fma_above
                                       ? pk_launch(k_tree_level<pk::kAddsFma>, grid, kTreeThreads, s, lv, pad, one)
                                       : pk_launch(k_tree_level<pk::kAddsPlain>, grid, kTreeThreads, s, lv, pad, one);
             if (e != cudaSuccess) return e;

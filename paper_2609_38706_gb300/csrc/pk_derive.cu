@@ -273,7 +273,6 @@ __device__ __forceinline__ void load_tables(uint32_t *sK, uint32_t *sPad, const 
 // ---------------------------------------------------------------------------
 constexpr int kDigestBlock = 128;
 constexpr int kStages = 3;
-constexpr uint32_t kFmaWarps = 3;  // warps of chunks per SM sub-partition from which kAddsFma is used
 
 constexpr int kRingRow = 20;  // words per thread and stage: 16, and 4 so that a quarter warp's 16-byte rows differ in bank
 typedef uint32_t RingStage[kDigestBlock][kRingRow];
@@ -1115,11 +1114,12 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
                           (const int64_t *)key_off, 0u, C, pad, keys, dw, one);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
-    // The multiply-add round form pays once at least kFmaWarps warps of chunks share each SM
-    // sub-partition (measured 10-13% per compression at 4 warps; slower for a lone warp).  The chunk
-    // count is at most key_capacity; with an unknown SM count the compiler's form is kept.
+    // The multiply-add round form pays once two warps of chunks share an SM sub-partition (two warps 4766 against
+    // 5191 cycles per compression each, a lone one 3170 against 2830; long-context key derivation, 1.7 warps per
+    // sub-partition, 870.7 -> 868.1 us).  The chunk count is at most key_capacity; with an unknown SM count the
+    // compiler's form is kept.
     const uint64_t warps = (key_capacity + 31) / 32;
-    const bool fma = ctx->sm_count > 0 && warps >= (uint64_t)kFmaWarps * 4u * ctx->sm_count;
+    const bool fma = ctx->sm_count > 0 && warps > 4ull * ctx->sm_count;
     const unsigned grid = grid_for(key_capacity, kDigestBlock) + dw.desc_blocks;
     // Few chunks: pairs of warps, at most three per SM, on the SMs that the descriptors and the offsets kernel, still
     // running when this launch comes up, leave free.  Key derivation of N chunks (8 per request), one lane per chunk |
