@@ -132,6 +132,14 @@ int pk_descriptor_encode(const pk_descriptor *desc, uint8_t *out, size_t cap, si
 int pk_descriptors_encode(const pk_descriptor *descs, uint32_t D, uint8_t *out, size_t cap,
                           int64_t *enc_off);
 
+/* Host.  The same for descriptors without appended dimensions whose fields lie
+ * back to back in registry order (model id, weight precision, weight version,
+ * adapter id, KV format, salt, of descriptor 0, then of descriptor 1, ...):
+ * field k of descriptor j has lens[6 j + k] bytes.  Same outputs and errors as
+ * pk_descriptors_encode; an encoding is at most 28 bytes longer than its fields. */
+int pk_descriptors_encode_packed(const uint8_t *fields, const uint32_t *lens, uint32_t D, uint8_t *out, size_t cap,
+                                 int64_t *enc_off);
+
 /* Host.  d = SHA-256(enc(canonical descriptor)) (Eq. 3, H over enc). */
 int pk_descriptor_digest(const pk_descriptor *desc, uint8_t out[32]);
 

@@ -231,6 +231,30 @@ int pk_descriptors_encode(const pk_descriptor *descs, uint32_t D, uint8_t *out, 
     return PK_OK;
 }
 
+int pk_descriptors_encode_packed(const uint8_t *fields, const uint32_t *lens, uint32_t D, uint8_t *out, size_t cap,
+                                 int64_t *enc_off) {
+    if (!enc_off || (D && (!fields || !lens))) return PK_ERR_ARG;
+    enc_off[0] = 0;
+    size_t pos = 0, at = 0;
+    std::string enc;
+    for (uint32_t j = 0; j < D; ++j) {
+        pk_bytes f[6];
+        for (int k = 0; k < 6; ++k) {
+            f[k].p = fields + at;
+            f[k].len = lens[6ull * j + k];
+            at += f[k].len;
+        }
+        const pk_descriptor d = {f[0], f[1], f[2], f[3], f[4], f[5], nullptr, 0};
+        const int rc = encode(&d, &enc);
+        if (rc != PK_OK) return rc;
+        if (pos + enc.size() > cap || !out) return PK_ERR_ARG;
+        std::memcpy(out + pos, enc.data(), enc.size());
+        pos += enc.size();
+        enc_off[j + 1] = (int64_t)pos;
+    }
+    return PK_OK;
+}
+
 int pk_descriptor_digest(const pk_descriptor *desc, uint8_t out[32]) {
     if (!out) return PK_ERR_ARG;
     std::string enc;

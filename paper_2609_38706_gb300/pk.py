@@ -82,6 +82,8 @@ def lib() -> ctypes.CDLL:
                                                     ctypes.POINTER(ctypes.c_size_t)]),
             "pk_descriptors_encode": (ctypes.c_int, [ctypes.POINTER(pk_descriptor), _U32, _VP,
                                                      ctypes.c_size_t, _VP]),
+            "pk_descriptors_encode_packed": (ctypes.c_int, [ctypes.c_char_p, ctypes.POINTER(_U32), _U32, _VP,
+                                                            ctypes.c_size_t, _VP]),
             "pk_descriptor_digest": (ctypes.c_int, [ctypes.POINTER(pk_descriptor), _VP]),
             "pk_worker_digest": (ctypes.c_int, [ctypes.POINTER(pk_descriptor), _VP]),
             "pk_request_digest": (ctypes.c_int, [_VP, ctypes.POINTER(pk_descriptor), _VP]),
@@ -230,13 +232,39 @@ def pk_descriptors_encode(descs, out: Optional[np.ndarray] = None,
     and ``enc_off`` (int64[D+1]).  Returns views (bytes used, offsets)."""
     d = _descs(descs)
     if out is None:
-        out = np.zeros(64 * 1024 + d.count * (7 * 4 + 8 * 4096), np.uint8)
+        out = np.zeros(encode_limit(d.count), np.uint8)
     if enc_off is None:
         enc_off = np.zeros(d.count + 1, np.int64)
     cap = out.numel() if isinstance(out, torch.Tensor) else out.size
     _check(lib().pk_descriptors_encode(d.array, d.count, _p(out), cap, _p(enc_off)), "pk_descriptors_encode")
     used = int(enc_off[d.count])
     return out[:used], enc_off
+
+
+def encode_limit(count: int) -> int:
+    """Bytes of the buffer that pk_descriptors_encode allocates for ``count`` descriptors."""
+    return 64 * 1024 + count * (7 * 4 + 8 * 4096)
+
+
+def pack_fields(descs: Iterable[Mapping]):
+    """(fields, lens, D) of descriptors without ``extra``, for
+    pk_descriptors_encode_packed; None if one of them has any."""
+    fields, n = [], 0
+    for d in descs:
+        if d.get("extra"):
+            return None
+        n += 1
+        for name in REGISTRY_V1:
+            v = d.get(name, b"")
+            fields.append(b"" if v is None else v.encode("utf-8") if isinstance(v, str) else bytes(v))
+    return b"".join(fields), (_U32 * len(fields))(*map(len, fields)), n
+
+
+def pk_descriptors_encode_packed(packed, out: int, cap: int, enc_off: int) -> None:
+    """Encode pack_fields' descriptors into the host memory at ``out`` (cap
+    bytes) with their offsets (int64[D+1]) at ``enc_off``."""
+    fields, lens, n = packed
+    _check(lib().pk_descriptors_encode_packed(fields, lens, n, out, cap, enc_off), "pk_descriptors_encode")
 
 
 def pk_descriptor_digest(desc) -> bytes:
@@ -335,12 +363,19 @@ def pk_derive_lookup_store(ctx: int, tokens: torch.Tensor, tok_off: torch.Tensor
                            enc: torch.Tensor, enc_off: torch.Tensor, digests: torch.Tensor, key_off: torch.Tensor,
                            keys: torch.Tensor, new_slots: torch.Tensor, hit_chunks: torch.Tensor, slots: torch.Tensor,
                            result: torch.Tensor, slot_out: torch.Tensor, status: torch.Tensor, stream=None) -> None:
+    derive_lookup_store_at(ctx, tokens, tok_off, desc_idx, _p(enc), enc.numel(), _p(enc_off), enc_off.numel() - 1, digests,
+                           key_off, keys, new_slots, hit_chunks, slots, result, slot_out, status, stream)
+
+
+def derive_lookup_store_at(ctx: int, tokens, tok_off, desc_idx, enc: Optional[int], enc_bytes: int, enc_off: Optional[int],
+                           D: int, digests, key_off, keys, new_slots, hit_chunks, slots, result, slot_out, status,
+                           stream=None) -> None:
+    """pk_derive_lookup_store with the D encodings given by address."""
     R = tok_off.numel() - 1
-    D = enc_off.numel() - 1
-    _check(lib().pk_derive_lookup_store(ctx, _p(tokens), tokens.numel(), _p(tok_off), R, _p(desc_idx), _p(enc),
-                                        enc.numel(), _p(enc_off), D, _p(digests), _p(key_off), _p(keys),
-                                        keys.numel() // 32, _p(new_slots), _p(hit_chunks), _p(slots), _p(result),
-                                        _p(slot_out), _p(status), _s(stream)), "pk_derive_lookup_store")
+    _check(lib().pk_derive_lookup_store(ctx, _p(tokens), tokens.numel(), _p(tok_off), R, _p(desc_idx), enc, enc_bytes,
+                                        enc_off, D, _p(digests), _p(key_off), _p(keys), keys.numel() // 32,
+                                        _p(new_slots), _p(hit_chunks), _p(slots), _p(result), _p(slot_out), _p(status),
+                                        _s(stream)), "pk_derive_lookup_store")
 
 
 def pk_compare_pages(slots: torch.Tensor, pages: torch.Tensor, ref_pages: torch.Tensor, verdict: torch.Tensor,
