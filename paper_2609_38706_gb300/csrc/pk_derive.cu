@@ -277,7 +277,8 @@ constexpr int kStages = 3;
 constexpr int kRingRow = 20;  // words per thread and stage: 16, and 4 so that a quarter warp's 16-byte rows differ in bank
 typedef uint32_t RingStage[kDigestBlock][kRingRow];
 
-// c = SHA-256 of chunk g (request r), written to keys[g].  F is the round
+// c = SHA-256 of chunk g (request r), written to keys[g] if `mine` (all 32
+// lanes call, those past the batch with its last chunk).  F is the round
 // form (pk_sha256.cuh: kAddsFma when several warps share each sub-partition).
 // Prompts packed back to back start at any 4-byte address: the ring then
 // holds the 16-byte aligned pieces that cover the chunk, and block b is read
@@ -289,7 +290,7 @@ template <int F>
 __device__ __forceinline__ void digest_chunk(const int32_t *tokens, const int64_t *tok_off,
                                              const int64_t *key_off, uint32_t r, int64_t g, uint32_t C,
                                              const uint32_t *sK, const uint32_t *sPad, RingStage *ring, uint8_t *keys,
-                                             uint32_t one) {
+                                             uint32_t one, bool mine) {
     const int64_t i = g - __ldcg(key_off + r);
     const int32_t *src = tokens + __ldcg(tok_off + r) + i * (int64_t)C;
     const uint32_t o = (uint32_t)(reinterpret_cast<uintptr_t>(src) & 15) / 4;  // the chunk's offset in its first 16 bytes
@@ -299,8 +300,8 @@ __device__ __forceinline__ void digest_chunk(const int32_t *tokens, const int64_
     pk::init_state(st);
     const uint32_t nfull = C / 16;
     uint32_t w[16];
-    if (base >= tokens) {
-        const bool shifted = __any_sync(__activemask(), o != 0);
+    if (__all_sync(0xffffffffu, base >= tokens)) {
+        const bool shifted = __any_sync(0xffffffffu, o != 0);
         // Pieces 0 .. nfull - 1 lie inside the chunk; of piece nfull the last block needs o words.
         auto load_piece = [&](uint32_t b, uint32_t stage) {
             if (b < nfull) cp_async_block(ring[stage][threadIdx.x], base + 16 * b);
@@ -368,7 +369,7 @@ __device__ __forceinline__ void digest_chunk(const int32_t *tokens, const int64_
             pk::compress_rolled<F>(st, w, sK, one);
         }
     }
-    store_digest(keys + 32 * g, st);
+    if (mine) store_digest(keys + 32 * g, st);
 }
 
 // Optional descriptor work for the same launch (fused a0): the first
@@ -411,16 +412,15 @@ k_chunk_digest(const int32_t *tokens, const int64_t *tok_off,
     pk::pdl_wait(tokens, tok_off, key_off, keys);
     if (R == 0) return;
     // all chunks, in tiles of one block, grid-strided
+    // (the warp index from a shuffle and the chunk clamped to the batch: uniform control flow, see lane_request_guess)
     const int64_t g_end = __ldcg(key_off + R);
     const uint32_t nblocks = gridDim.x - dw.desc_blocks;
-    for (int64_t tile = (int64_t)(blockIdx.x - dw.desc_blocks) * kDigestBlock; tile < g_end;
-         tile += (int64_t)nblocks * kDigestBlock) {
-        const int64_t g = tile + threadIdx.x;
-        const int64_t g0 = g - (threadIdx.x & 31);
-        if (g0 >= g_end) break;  // whole warp past the end (uniform per warp)
+    const uint32_t warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    for (int64_t g0 = (int64_t)(blockIdx.x - dw.desc_blocks) * kDigestBlock + 32 * warp; g0 < g_end;
+         g0 += (int64_t)nblocks * kDigestBlock) {
+        const int64_t g = g0 + lane < g_end ? g0 + lane : g_end - 1;
         const uint32_t r = pk::lane_request_guess(key_off, R, g0, g_end, g);
-        if (g < g_end) digest_chunk<F>(tokens, tok_off, key_off, r, g, C, sK, sPad, ring, keys, one);
-        __syncwarp();
+        digest_chunk<F>(tokens, tok_off, key_off, r, g, C, sK, sPad, ring, keys, one, g0 + lane < g_end);
     }
     pk::pdl_launch_dependents();
 }

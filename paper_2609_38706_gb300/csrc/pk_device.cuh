@@ -59,57 +59,72 @@ __device__ __forceinline__ uint32_t lane_request(const int64_t *key_off, uint32_
     return find_request_in(key_off, r0, r1 + 1, g < total ? g : total - 1);
 }
 
-// Same result as lane_request with one search: r0 (the request of the warp's
-// first item) by warp_find_request, then one 32-wide load of key_off[r0+1 ..]
-// and a search over those 32 values by shuffles (non-decreasing key_off: r = r0
-// + the count of them <= g, one of 33 outcomes: 6 halvings).  A lane whose item
-// lies past those 32 requests (only after runs of empty requests) falls back to
-// find_request_in.
-__device__ __forceinline__ uint32_t lane_request_window(const int64_t *key_off, uint32_t R, int64_t g0,
-                                                        int64_t total, int64_t g) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t r0 = warp_find_request(key_off, R, g0);
-    const uint64_t p = (uint64_t)r0 + 1 + lane;
-    const int64_t v = p <= R ? __ldcg(key_off + p) : INT64_MAX;
-    const int64_t gg = g < total ? g : total - 1;
-    int lo = 0, hi = 32;  // the first j with key_off[r0 + 1 + j] > gg lies in [lo, hi] (32: none of the 32)
-#pragma unroll
-    for (int it = 0; it < 6; ++it) {
-        const int mid = (lo + hi) >> 1;
-        const int64_t vm = __shfl_sync(0xffffffffu, v, mid < 31 ? mid : 31);
-        if (lo < hi) {
-            if (vm <= gg) lo = mid + 1; else hi = mid;
-        }
-    }
-    if (lo < 32) return r0 + (uint32_t)lo;
-    return find_request_in(key_off, r0 + 32, R, gg);
-}
-
-// Same result again, for batches of about equal requests: a guess from the mean
-// request size, r_g = g0 * R / total, one 32-wide load of key_off[w0 ..] with
-// w0 = r_g - 8, and the same shuffle search; used when that window brackets
-// every lane's item, else lane_request_window.
+// Same result as lane_request, in code whose control flow is uniform over the
+// warp as far as the compiler can see: every branch is on a vote and every loop
+// runs a number of times that follows from R alone.  A loop or branch that may
+// diverge, even one that never runs, costs the code after it the uniform data
+// path (the chunk digests of batches of equal requests, whose mapping never
+// left its first lines: with divergent searches in the fallback and a divergent
+// end of the batch, sweep key derivation 207 us, small-block 613.8; 196.5 and
+// 591.9 so).
+//
+// First a guess for batches of about equal requests, r_g = g0 * R / total, and
+// one 32-wide load of key_off[w0 ..], w0 = r_g - 8.  With p_j = key_off[w0 + j] -
+// g0 clamped to 0..32, item g0 + l lies in request w0 + (number of p_j <= l) - 1:
+// the p_j = 0 by a ballot, the others by a mask of their positions when they
+// differ (no empty requests among them).  When the window does not bracket the
+// warp's items, or requests in it are empty: a 32-ary search for the request r0
+// of the first item, the same window from r0 counted by a search over shuffles,
+// and for items past those 32 requests (after runs of empty ones) a binary
+// search of key_off.
 __device__ __forceinline__ uint32_t lane_request_guess(const int64_t *key_off, uint32_t R, int64_t g0,
                                                        int64_t total, int64_t g) {
+    constexpr uint32_t kFull = 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31;
     const int64_t gg = g < total ? g : total - 1;
+    const uint32_t l = (uint32_t)(gg - g0);  // this lane's item, 0..31
+    auto window = [&](uint32_t w0) {         // p of key_off[w0 + lane]
+        const uint64_t at = (uint64_t)w0 + lane;
+        const int64_t d = (at <= R ? __ldcg(key_off + at) : INT64_MAX) - g0;
+        return d <= 0 ? 0u : d > 31 ? 32u : (uint32_t)d;
+    };
+    const uint32_t last = total - g0 < 32 ? (uint32_t)(total - g0) - 1 : 31u;
     uint32_t rg = (uint32_t)((float)g0 / (float)total * (float)R);
     rg = rg >= R ? R - 1 : rg;
     const uint32_t w0 = rg > 8 ? rg - 8 : 0;
-    const uint64_t p = (uint64_t)w0 + lane;
-    const int64_t u = p <= R ? __ldcg(key_off + p) : INT64_MAX;
-    const int64_t u0 = __shfl_sync(0xffffffffu, u, 0);
-    int lo = 1, hi = 32;  // the first j >= 1 with key_off[w0 + j] > gg lies in [lo, hi] (32: none of the 31)
-#pragma unroll
-    for (int it = 0; it < 6; ++it) {
-        const int mid = (lo + hi) >> 1;
-        const int64_t vm = __shfl_sync(0xffffffffu, u, mid < 31 ? mid : 31);
-        if (lo < hi) {
-            if (vm <= gg) lo = mid + 1; else hi = mid;
-        }
+    uint32_t p = window(w0);
+    const uint32_t before = __ballot_sync(kFull, p == 0), among = __ballot_sync(kFull, p - 1 < 31);
+    const uint32_t places = __reduce_or_sync(kFull, p - 1 < 31 ? 1u << p : 0u);
+    if ((before & 1u) && __ballot_sync(kFull, p > last) && __popc(places) == __popc(among))
+        return w0 + __popc(before) - 1 + __popc(places & ((2u << l) - 1u));
+    // the request r0 of item g0: blocks of `step` requests, the last one that starts at or before g0
+    uint32_t r0 = 0;
+    for (uint32_t span = R; span > 1;) {
+        const uint32_t step = (span + 31) / 32;
+        const uint64_t c = (uint64_t)r0 + (uint64_t)(lane + 1) * step;
+        r0 += step * __popc(__ballot_sync(kFull, c < R && __ldcg(key_off + c) <= g0));
+        span = step;
     }
-    if (__all_sync(0xffffffffu, u0 <= g0 && lo < 32)) return w0 + (uint32_t)lo - 1;
-    return lane_request_window(key_off, R, g0, total, g);
+    // items within the 32 requests from r0: the number of boundaries among key_off[r0 + 1 ..] at or before the item
+    p = window(r0 + 1);
+    uint32_t lo = 0, hi = 32;
+#pragma unroll 1
+    for (int it = 0; it < 6; ++it) {
+        const uint32_t mid = (lo + hi) >> 1;
+        const uint32_t pm = __shfl_sync(kFull, p, mid < 31 ? mid : 31);
+        const bool up = lo < hi && pm <= l;
+        hi = lo < hi && !up ? mid : hi;
+        lo = up ? mid + 1 : lo;
+    }
+    if (__all_sync(kFull, lo < 32)) return r0 + lo;
+    uint32_t r = r0;
+#pragma unroll 1
+    for (uint32_t n = R - r0; n > 1;) {  // the last request of the n from r that starts at or before the item
+        const uint32_t h = n >> 1;
+        r = __ldcg(key_off + r + h) <= gg ? r + h : r;
+        n -= h;
+    }
+    return r;
 }
 
 }  // namespace pk
