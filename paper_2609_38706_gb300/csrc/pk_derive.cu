@@ -535,6 +535,14 @@ k_chunk_digest_pairs(const int32_t *tokens, const int64_t *tok_off, const int64_
 // ---------------------------------------------------------------------------
 constexpr int kChainLanes = 32;
 
+// The largest n >= 0 of the warp, by reductions whose result the compiler knows to be uniform (see
+// lane_request_guess: the chains' loops over it then count in uniform registers).
+__device__ __forceinline__ int64_t warp_max(int64_t n) {
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)((uint64_t)n >> 32));
+    const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)((uint64_t)n >> 32) == hi ? (uint32_t)n : 0u);
+    return (int64_t)((uint64_t)hi << 32 | lo);
+}
+
 __device__ __forceinline__ void bar_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
 
@@ -588,9 +596,10 @@ __device__ __forceinline__ void rounds16_kw(uint32_t v[8], const uint4 (*kw)[kCh
 // schedule warp p + 4, which share a sub-partition: the schedule fills the issue slots that the rounds warp's
 // dependency chain leaves idle.
 // FS1, FS2: the forms (pk_sha256.cuh) of the schedule warp's additions for block 1 and block 2, `one` their
-// run-time 1.  The rounds warp keeps the compiler's form: its dependency chain sets the step time, and a
-// multiply-add's longer latency there made the chain slower (small-block key derivation 674 -> 718 us with
-// every addition on the FMA pipe).  The schedule warp's two blocks differ:
+// run-time 1.  The rounds warp's dependency chain sets the step time, and a multiply-add's longer latency there made
+// the chain slower (small-block key derivation 674 -> 718 us with every addition on the FMA pipe); it takes the late
+// form, one add on the ALU after the rotations (580.9 -> 572.5 us against the compiler's form; both with uniform
+// loops and warp roles, without them 605.4 and 613.9).  The schedule warp's two blocks differ:
 // block 1's schedule (k_{i-1} || d) can start only when k_{i-1} is published, and the rounds warp waits for
 // it after its 16th round, so it keeps the short-latency form; block 2's (c_i || padding) is made a step
 // ahead, off the critical path, and its additions go to the FMA pipe, where they do not compete with the
@@ -608,7 +617,7 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
         const uint8_t *digests, uint32_t R, uint32_t D, uint8_t *keys, uint32_t groups, uint32_t one) {
     extern __shared__ __align__(16) uint8_t chain_smem[];
     pk::pdl_wait(key_off, desc_idx, digests, keys);  // successor released at the last step (see k_chunk_digest)
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     const uint32_t pair = warp & (kChainPairs - 1);
     const bool sched = warp >= (uint32_t)kChainPairs;
     ChainSmem &sm = reinterpret_cast<ChainSmem *>(chain_smem)[pair];
@@ -628,12 +637,7 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
         di = desc_idx[r];
         if (n < 0 || di >= D) n = 0;
     }
-    int64_t nmax = n;  // identical in both warps of the pair: they cover the same 32 requests
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int64_t x = __shfl_xor_sync(0xffffffffu, nmax, o);
-        nmax = x > nmax ? x : nmax;
-    }
+    const int64_t nmax = warp_max(n);  // identical in both warps of the pair: they cover the same requests
     if (nmax == 0) {  // uniform over the pair
         pk::pdl_launch_dependents();
         __syncthreads();
@@ -726,23 +730,23 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
         {   // block 1, rounds 0..15: W = k_{i-1} || d
             uint32_t a_ = v[0], b_ = v[1], c_ = v[2], d_ = v[3], e_ = v[4], f_ = v[5], g_ = v[6], h_ = v[7];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) pk::round_kw(a_, b_, c_, d_, e_, f_, g_, h_, pk::kSha256K[j] + p[j]);
+            for (int j = 0; j < 8; ++j) pk::round_kw<pk::kAddsLate>(a_, b_, c_, d_, e_, f_, g_, h_, pk::kSha256K[j] + p[j], one);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) pk::round_kw(a_, b_, c_, d_, e_, f_, g_, h_, kd[j]);
+            for (int j = 0; j < 8; ++j) pk::round_kw<pk::kAddsLate>(a_, b_, c_, d_, e_, f_, g_, h_, kd[j], one);
             v[0] = a_; v[1] = b_; v[2] = c_; v[3] = d_; v[4] = e_; v[5] = f_; v[6] = g_; v[7] = h_;
         }
         bar_sync(bar_s1);
-        rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 1, lane, one);
+        rounds16_kw<pk::kAddsLate>(v, sm.kw1, 1, lane, one);
         bar_sync(bar_s1b);
-        rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 2, lane, one);
-        rounds16_kw<pk::kAddsPlain>(v, sm.kw1, 3, lane, one);
+        rounds16_kw<pk::kAddsLate>(v, sm.kw1, 2, lane, one);
+        rounds16_kw<pk::kAddsLate>(v, sm.kw1, 3, lane, one);
         uint32_t st[8] = {PK_IV0 + v[0], PK_IV1 + v[1], PK_IV2 + v[2], PK_IV3 + v[3],
                           PK_IV4 + v[4], PK_IV5 + v[5], PK_IV6 + v[6], PK_IV7 + v[7]};
         const uint4 (*kw2)[kChainLanes] = sm.kw2[i & 1];
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = st[j];
 #pragma unroll 1
-        for (int q = 0; q < 4; ++q) rounds16_kw<pk::kAddsPlain>(v, kw2, q, lane, one);
+        for (int q = 0; q < 4; ++q) rounds16_kw<pk::kAddsLate>(v, kw2, q, lane, one);
 #pragma unroll
         for (int j = 0; j < 8; ++j) p[j] = st[j] + v[j];
         if (i < n) store_digest(keys + 32ull * (a + i), p);
@@ -847,12 +851,7 @@ k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *d
         di = desc_idx[r];
         if (n < 0 || di >= D) n = 0;
     }
-    int64_t nmax = n;  // identical in both warps of the pair: they cover the same requests
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int64_t x = __shfl_xor_sync(0xffffffffu, nmax, o);
-        nmax = x > nmax ? x : nmax;
-    }
+    const int64_t nmax = warp_max(n);  // identical in both warps of the pair: they cover the same requests
     if (nmax == 0) {  // uniform over the pair
         pk::pdl_launch_dependents();
         if (kPairs > 1) __syncthreads();

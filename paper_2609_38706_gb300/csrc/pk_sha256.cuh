@@ -218,8 +218,12 @@ namespace pk {
 //               run-time 1 the compiler cannot fold): 22.2 cycles per round
 //               and 10-13% faster compressions once 4 or more warps share a
 //               sub-partition, but 33.4 cycles for a lone warp (the
-//               multiply-add's longer latency sits on the critical path).
-enum { kAddsPlain = 0, kAddsFma = 1 };
+//               multiply-add's longer latency sits on the critical path);
+//   kAddsLate   (rounds only) one 3-input add after each set of rotations,
+//               e' = S1 + Ch + (d + h + kw) and a' = e' + S0 + (Maj - d), the
+//               sums in brackets made beside them, two of them on the FMA pipe:
+//               for a warp that shares its sub-partition with one other.
+enum { kAddsPlain = 0, kAddsFma = 1, kAddsLate = 2 };
 
 // x * one + c, kept as a multiply-add (one == 1 at run time).
 __device__ __forceinline__ uint32_t mad1(uint32_t x, uint32_t one, uint32_t c) {
@@ -241,6 +245,12 @@ __device__ __forceinline__ void round_kw(uint32_t &a, uint32_t &b, uint32_t &c, 
         const uint32_t t1 = mad1(big_s1(e), one, mad1(ch(e, f, g), one, mad1(h, one, kw)));
         const uint32_t t2 = mad1(big_s0(a), one, maj(a, b, c));
         h = g; g = f; f = e; e = mad1(d, one, t1); d = c; c = b; b = a; a = mad1(t1, one, t2);
+    } else if (F == kAddsLate) {
+        uint32_t t = h + kw;
+        asm("" : "+r"(t));  // (kept apart from the late sum)
+        const uint32_t e1 = big_s1(e) + ch(e, f, g) + mad1(d, one, t);
+        const uint32_t a1 = e1 + big_s0(a) + mad1(d, 0u - one, maj(a, b, c));
+        h = g; g = f; f = e; e = e1; d = c; c = b; b = a; a = a1;
     } else {
         const uint32_t t1 = h + big_s1(e) + ch(e, f, g) + kw;
         const uint32_t t2 = big_s0(a) + maj(a, b, c);
