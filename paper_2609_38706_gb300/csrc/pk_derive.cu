@@ -118,22 +118,44 @@ k_digest_descriptors(const uint8_t *enc, uint64_t enc_bytes, const int64_t *enc_
 }
 
 // ---------------------------------------------------------------------------
-// Chunk offsets: one block, requests in tiles of kScanThreads * kScanItems.
-// Each thread takes kScanItems consecutive requests of the tile (coalesced
-// offset loads), the block scans the per-thread sums, and a running carry
-// links the tiles.  Any invalid request (offsets decreasing, negative or past
-// n_tokens, descriptor index >= D) or a total above key_capacity zeroes all
-// offsets afterwards and reports PK_ERR_ARG.
+// Chunk offsets: one block per tile of kScanThreads * kScanItems requests.
+// Each block scans its own tile (kScanItems consecutive requests per thread)
+// and sums the requests of every other tile with independent, coalesced loads:
+// those before it give its first offset, all of them the checks.  That is more
+// loads, but no block waits for another and none walks the tiles one after the
+// other (key derivation of 16,384 prompts of 32 tokens 37.6 -> 29.1 us, of 100,000
+// 171 -> 100 us).  Any invalid request (offsets
+// decreasing, negative or past n_tokens, descriptor index >= D) or a total
+// above key_capacity makes all offsets zero and reports PK_ERR_ARG.
 // ---------------------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
+constexpr uint32_t kScanTile = kScanThreads * kScanItems;
 
+// Full chunks of the request [a, b) with descriptor index di; bad is set if it is invalid.
+__device__ __forceinline__ long long request_chunks(int64_t a, int64_t b, uint32_t di, uint64_t n_tokens, uint32_t C,
+                                                    uint32_t D, bool &bad) {
+    if (a < 0 || b < a || (uint64_t)b > n_tokens || di >= D) {
+        bad = true;
+        return 0;
+    }
+    const uint64_t len = (uint64_t)(b - a);  // 32-bit division when the request fits (64-bit is a long library sequence)
+    return len >> 32 ? (long long)(len / C) : (long long)((uint32_t)len / C);
+}
+
+__device__ __forceinline__ long long warp_sum(long long x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+template <bool kTiles>  // false: one tile
 __global__ void __launch_bounds__(kScanThreads)
 k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t C,
                 const uint32_t *desc_idx, uint32_t D, uint64_t key_capacity,
                 int64_t *key_off, int32_t *status) {
-    __shared__ long long warp_sums[kScanThreads / 32];
-    __shared__ long long tile_total;
+    __shared__ long long warp_sums[kScanThreads / 32], warp_before[kScanThreads / 32], warp_after[kScanThreads / 32];
+    __shared__ long long sh_total;
     pk::pdl_wait(tok_off, desc_idx, key_off, status);
     // The chunk digests are released only here, when every earlier kernel of the stream is done: released at the
     // start, their CTAs came up beside the previous batch's last kernels and stacked on the SMs those left free,
@@ -142,82 +164,81 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
     // context 1056 -> 947 us (both sides with the two-lane chain).
     pk::pdl_launch_dependents();
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0) key_off[0] = 0;
+    const uint64_t base = (uint64_t)blockIdx.x * kScanTile, r0 = base + (uint64_t)tid * kScanItems;
     bool bad = false;
-    long long carry = 0;
-    // a tile's inputs (its threads' tok_off[r0 .. r0 + kScanItems], desc_idx[r0 .. r0 + kScanItems)) are loaded
-    // one tile ahead, so that they are in flight during the previous tile's scan
-    constexpr uint64_t kTile = (uint64_t)kScanThreads * kScanItems;
-    int64_t to_cur[kScanItems + 1], to_nxt[kScanItems + 1] = {};
-    uint32_t di_cur[kScanItems], di_nxt[kScanItems] = {};
-    auto load_tile = [&](uint64_t base, int64_t *to, uint32_t *di) {
-        const uint64_t r0 = base + (uint64_t)tid * kScanItems;
+    int64_t to[kScanItems + 1];
+    uint32_t di[kScanItems];
 #pragma unroll
-        for (int j = 0; j <= kScanItems; ++j) to[j] = r0 + j <= R ? tok_off[r0 + j] : 0;
+    for (int j = 0; j <= kScanItems; ++j) to[j] = r0 + j <= R ? tok_off[r0 + j] : 0;
 #pragma unroll
-        for (int j = 0; j < kScanItems; ++j) di[j] = r0 + j < R ? desc_idx[r0 + j] : 0u;
-    };
-    if (R > 0) load_tile(0, to_cur, di_cur);
-    for (uint64_t base = 0; base < R; base += kTile) {
-        if (base + kTile < R) load_tile(base + kTile, to_nxt, di_nxt);
-        const uint64_t r0 = base + (uint64_t)tid * kScanItems;
-        long long n[kScanItems];
-        long long local = 0;
+    for (int j = 0; j < kScanItems; ++j) di[j] = r0 + j < R ? desc_idx[r0 + j] : 0u;
+    long long before = 0, after = 0;  // chunks of the tiles before and after this one
+    for (uint64_t other = 0; kTiles && other < R; other += kScanTile) {
+        if (other == base) continue;
+        int64_t a[kScanItems], b[kScanItems];
+        uint32_t d[kScanItems];
 #pragma unroll
         for (int j = 0; j < kScanItems; ++j) {
-            const uint64_t r = r0 + j;
-            n[j] = 0;
-            if (r < R) {
-                const int64_t a = to_cur[j], b = to_cur[j + 1];
-                if (a < 0 || b < a || (uint64_t)b > n_tokens || di_cur[j] >= D) {
-                    bad = true;
-                } else {  // 32-bit division when the request fits (64-bit division is a long library sequence)
-                    const uint64_t len = (uint64_t)(b - a);
-                    n[j] = len >> 32 ? (long long)(len / C) : (long long)((uint32_t)len / C);
-                }
-            }
-            local += n[j];
+            const uint64_t r = other + j * kScanThreads + tid;
+            a[j] = r < R ? tok_off[r] : 0;
+            b[j] = r < R ? tok_off[r + 1] : 0;
+            d[j] = r < R ? desc_idx[r] : 0u;
         }
-        // block exclusive scan of the per-thread sums
-        long long incl = local;
+        long long sum = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
+        for (int j = 0; j < kScanItems; ++j)
+            if (other + j * kScanThreads + tid < R) sum += request_chunks(a[j], b[j], d[j], n_tokens, C, D, bad);
+        if (other < base) before += sum;
+        else after += sum;
+    }
+    long long n[kScanItems];
+    long long local = 0;
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) {
+        n[j] = r0 + j < R ? request_chunks(to[j], to[j + 1], di[j], n_tokens, C, D, bad) : 0;
+        local += n[j];
+    }
+    // block exclusive scan of the per-thread sums, and the other tiles' totals
+    long long incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) warp_sums[warp] = incl;
+    if (kTiles) {
+        before = warp_sum(before);
+        after = warp_sum(after);
+        if (lane == 0) {
+            warp_before[warp] = before;
+            warp_after[warp] = after;
         }
-        if (lane == 31) warp_sums[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const long long ws = warp_sums[lane];
-            long long wincl = ws;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long v = __shfl_up_sync(0xffffffffu, wincl, o);
-                if (lane >= o) wincl += v;
-            }
-            warp_sums[lane] = wincl - ws;
-            if (lane == 31) tile_total = wincl;
-        }
-        __syncthreads();
-        long long run = carry + warp_sums[warp] + incl - local;
-#pragma unroll
-        for (int j = 0; j < kScanItems; ++j) {
-            if (r0 + j < R) {
-                run += n[j];
-                key_off[r0 + j + 1] = run;
-            }
-        }
-        carry += tile_total;
-        __syncthreads();  // warp_sums and tile_total are reused by the next tile
-#pragma unroll
-        for (int j = 0; j <= kScanItems; ++j) to_cur[j] = to_nxt[j];
-#pragma unroll
-        for (int j = 0; j < kScanItems; ++j) di_cur[j] = di_nxt[j];
     }
     bad = __syncthreads_or(bad);
-    if (bad || (unsigned long long)carry > key_capacity) {
-        for (uint64_t r = tid; r < R; r += kScanThreads) key_off[r + 1] = 0;
-        if (tid == 0) set_status(status, PK_ERR_ARG);
+    if (warp == 0) {
+        const long long ws = warp_sums[lane];
+        long long wincl = ws;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long v = __shfl_up_sync(0xffffffffu, wincl, o);
+            if (lane >= o) wincl += v;
+        }
+        const long long first = kTiles ? warp_sum(warp_before[lane]) : 0;
+        const long long rest = kTiles ? warp_sum(warp_after[lane]) : 0;
+        warp_sums[lane] = first + wincl - ws;
+        if (lane == 31) sh_total = first + wincl + rest;
+    }
+    __syncthreads();
+    bad |= (unsigned long long)sh_total > key_capacity;
+    long long run = warp_sums[warp] + incl - local;
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) {
+        run += n[j];
+        if (r0 + j < R) key_off[r0 + j + 1] = bad ? 0 : run;
+    }
+    if (blockIdx.x == 0 && tid == 0) {
+        key_off[0] = 0;
+        if (bad) set_status(status, PK_ERR_ARG);
     }
 }
 
@@ -1096,8 +1117,9 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     static_assert(kDigestBlock / 32 * kDescStage <= (int)sizeof(RingStage) * kStages,
                   "descriptor staging fits in the token ring");
     const uint32_t C = ctx->chunk_tokens;
-    cudaError_t e = pk_launch(k_chunk_offsets, 1, kScanThreads, s, tok_off, R, n_tokens, C, desc_idx, D, key_capacity,
-                              key_off, status);
+    cudaError_t e = pk_launch(R <= kScanTile ? k_chunk_offsets<false> : k_chunk_offsets<true>,
+                              R <= kScanTile ? 1 : grid_for(R, kScanTile), kScanThreads, s, tok_off, R, n_tokens, C,
+                              desc_idx, D, key_capacity, key_off, status);
     if (e != cudaSuccess) return e;
     DescWork dw = {enc, enc_bytes, enc_off, D, digests, status, 0};
     if (enc_off) dw.desc_blocks = grid_for(D, kDigestBlock / 32);
