@@ -387,7 +387,8 @@ k_first_miss(const int64_t *key_off, uint32_t R, uint64_t key_capacity,
 // mode), [1] requests handed out by a work-taking lookup-and-store, [2]
 // entries deferred in this call, [3] keys its claims claimed, [4] keys its
 // admission pass claimed, [5] CTAs of the claim kernel done (reset by the
-// last); the finalize kernel adds [3] and [4] to [0] and clears [2..4].
+// last), [6] whether the call claimed a key (set by the last); the finalize
+// kernel adds [3] and [4] to [0] and clears [2..4].
 // ---------------------------------------------------------------------------
 enum Examine { kAdvance, kDone, kClaimedHere };
 enum ClaimMode : uint32_t {
@@ -764,13 +765,15 @@ __device__ __noinline__ void store_admit(pk_entry *table, uint64_t mask, uint32_
 
 // End of a claim kernel: the last CTA to finish (every CTA counts itself on
 // counter[5] after a fence) runs the admission pass when the call deferred
-// entries, and resets counter[5] for the next call.  Every CTA of the grid
-// must call it.
+// entries, resets counter[5] for the next call, and sets *any_new (if given) to
+// whether the call claimed a key: without one no entry is PENDING.  Every CTA
+// of the grid must call it.
 __device__ __forceinline__ void admit_if_last(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t capacity,
                                               unsigned long long *counter, unsigned long long epoch,
                                               unsigned long long *stamps, const uint8_t *keys, const uint32_t *slots,
                                               uint64_t n, const int64_t *key_off, uint32_t R, int32_t *result,
-                                              uint32_t *slot_out, uint32_t *pos_out, int32_t *status) {
+                                              uint32_t *slot_out, uint32_t *pos_out, int32_t *status,
+                                              unsigned long long *any_new) {
     __shared__ int s_last;
     __threadfence();  // this CTA's results and counts are visible to the GPU before it counts itself
     __syncthreads();
@@ -779,9 +782,15 @@ __device__ __forceinline__ void admit_if_last(pk_entry *table, uint64_t mask, ui
     if (!s_last) return;
     __threadfence();
     if (threadIdx.x == 0) counter[5] = 0;
-    if (__ldcg(counter + 2) == 0) return;  // nothing deferred: the claim kernel decided every entry
-    store_admit(table, mask, max_probe, capacity, counter, epoch, stamps, keys, slots, n, key_off, R, result,
-                slot_out, pos_out, status);
+    const unsigned long long deferred = __ldcg(counter + 2);
+    unsigned long long claimed = __ldcg(counter + 3);
+    if (deferred) {  // else the claim kernel decided every entry
+        store_admit(table, mask, max_probe, capacity, counter, epoch, stamps, keys, slots, n, key_off, R, result,
+                    slot_out, pos_out, status);
+        __syncthreads();  // the admission pass has added its claims
+        claimed |= __ldcg(counter + 4);
+    }
+    if (threadIdx.x == 0 && any_new) *any_new = claimed != 0ull;
 }
 
 // List mode, or range mode for few long requests: one warp per 32
@@ -819,7 +828,7 @@ k_store_claim(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t capac
     pk::pdl_launch_dependents();
     count_claims(block_sums, claims, e < n && res == PK_STORE_DEFERRED, counter);
     admit_if_last(table, mask, max_probe, capacity, counter, epoch, stamps, keys, slots, n, key_off, R, result, slot_out,
-                  slot_out, status);
+                  slot_out, status, counter + 6);
 }
 
 // Range mode for many short requests: one warp per request, no search.
@@ -906,7 +915,7 @@ k_store_claim_req(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t c
     pk::pdl_launch_dependents();
     count_claims(block_sums, claims, deferred, counter);
     admit_if_last(table, mask, max_probe, capacity, counter, epoch, stamps, keys, slots, n, key_off, R, result, slot_out,
-                  slot_out, status);
+                  slot_out, status, counter + 6);
 }
 
 // ---------------------------------------------------------------------------
@@ -1047,7 +1056,7 @@ k_lookup_store_req(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t 
     }
     count_claims(block_sums, claims, deferred, counter);
     admit_if_last(table, mask, max_probe, capacity, counter, epoch, stamps, keys, new_slots, key_capacity, key_off, R,
-                  result, slot_out, slot_out, status);
+                  result, slot_out, slot_out, status, counter + 6);
 }
 
 // Few long requests: one warp per 32 consecutive keys; k_lookup_store_tail
@@ -1088,7 +1097,7 @@ k_lookup_store(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t capa
     pk::pdl_launch_dependents();
     count_claims(block_sums, claims, e < end && res == PK_STORE_DEFERRED, counter);
     admit_if_last(table, mask, max_probe, capacity, counter, epoch, stamps, keys, new_slots, key_capacity, key_off, R,
-                  result, slot_out, slot_out, status);
+                  result, slot_out, slot_out, status, counter + 6);
 }
 
 // One warp per request: h_r = the first miss (slot PK_NO_SLOT), entries below
@@ -1129,14 +1138,22 @@ k_lookup_store_tail(const int64_t *key_off, uint32_t R, uint64_t key_capacity,
 // final once every claim is in: the lowest claimant is INSERTED, the others
 // PRESENT with its slot.  In range mode, entries past key_off[R] (not keys
 // of this batch) are skipped.  The call's claims are added to the entry
-// count, and its counter words [2..4] cleared.
+// count, and its counter words [2..4] cleared.  counter[6] says whether the
+// call claimed a key at all: in a call that did not (every key found) a thread
+// leaves after its first loads.  kItems entries per thread, their loads in
+// flight together: four for calls of more entries than the SMs hold threads
+// (small-block lookup and store, 2.1 M keys all found: 100.6 us with one, 91.2
+// with four), one below (262,144 inserts: four cost 1.3 us more).
+template <uint32_t kItems>
 __global__ void __launch_bounds__(256)
 k_store_finalize(const pk_entry *table, uint64_t n, const int64_t *key_off, uint32_t R,
                  int32_t *result, uint32_t *slot_out, unsigned long long *counter) {
     pk::pdl_launch_dependents();
     pk::pdl_wait(table, key_off, result, slot_out, counter);
-    const uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e == 0) {
+    const bool any_new = __ldcg(counter + 6) != 0ull;
+    const uint64_t total = key_off ? (R > 0 ? (uint64_t)__ldcg(key_off + R) : 0ull) : n;
+    const uint64_t e0 = (uint64_t)blockIdx.x * (blockDim.x * kItems) + threadIdx.x;
+    if (e0 == 0) {
         const unsigned long long c2 = __ldcg(counter + 2), c3 = __ldcg(counter + 3), c4 = __ldcg(counter + 4);
         if (c3 | c4) counter[0] += c3 + c4;
         if (c2 | c3 | c4) {
@@ -1145,16 +1162,31 @@ k_store_finalize(const pk_entry *table, uint64_t n, const int64_t *key_off, uint
             counter[4] = 0;
         }
     }
-    if (e >= n) return;
-    if (key_off && (int64_t)e >= (R > 0 ? __ldcg(key_off + R) : 0)) {
-        result[e] = PK_STORE_SKIPPED;
-        slot_out[e] = PK_NO_SLOT;
-        return;
+    int32_t res[kItems];  // (read beside the words above)
+#pragma unroll
+    for (uint32_t u = 0; u < kItems; ++u) {
+        const uint64_t e = e0 + u * blockDim.x;
+        res[u] = e < n ? result[e] : PK_STORE_SKIPPED;
     }
-    if (result[e] != PK_STORE_PENDING) return;
-    const unsigned long long w = *reinterpret_cast<const unsigned long long *>(&table[slot_out[e]].slot);
-    result[e] = ~(uint32_t)(w >> 32) == (uint32_t)e ? PK_STORE_INSERTED : PK_STORE_PRESENT;
-    slot_out[e] = (uint32_t)w;
+    if (!any_new && e0 + blockDim.x * (kItems - 1) < total) return;
+    uint32_t pos[kItems];
+#pragma unroll
+    for (uint32_t u = 0; u < kItems; ++u) pos[u] = any_new && res[u] == PK_STORE_PENDING ? slot_out[e0 + u * blockDim.x] : 0u;
+    unsigned long long w[kItems];
+#pragma unroll
+    for (uint32_t u = 0; u < kItems; ++u)
+        w[u] = any_new && res[u] == PK_STORE_PENDING ? *reinterpret_cast<const unsigned long long *>(&table[pos[u]].slot) : 0ull;
+#pragma unroll
+    for (uint32_t u = 0; u < kItems; ++u) {
+        const uint64_t e = e0 + u * blockDim.x;
+        if (e >= total && e < n) {
+            result[e] = PK_STORE_SKIPPED;
+            slot_out[e] = PK_NO_SLOT;
+        } else if (any_new && res[u] == PK_STORE_PENDING) {
+            result[e] = ~(uint32_t)(w[u] >> 32) == (uint32_t)e ? PK_STORE_INSERTED : PK_STORE_PRESENT;
+            slot_out[e] = (uint32_t)w[u];
+        }
+    }
 }
 
 // Table load from device memory in one pass: each 32-byte entry copied whole
@@ -1276,7 +1308,7 @@ k_noalloc_claim(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t cap
     }
     count_claims(block_sums, claims, e < n && res == PK_STORE_DEFERRED, sc->word);
     admit_if_last(table, mask, max_probe, capacity, sc->word, epoch, nullptr, keys, slots, n, key_off, R, result,
-                  slot_out, sc->pos, status);
+                  slot_out, sc->pos, status, nullptr);
 }
 
 __global__ void __launch_bounds__(256)
@@ -1356,6 +1388,13 @@ cudaError_t pk_launch_lookup(const pk_ctx *ctx, const uint8_t *keys, const int64
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+static cudaError_t launch_finalize(const pk_ctx *ctx, uint64_t n, const int64_t *key_off, uint32_t R, int32_t *result,
+                                   uint32_t *slot_out, cudaStream_t s) {
+    const bool many = n > 2048ull * ctx->sm_count;
+    return pk_launch(many ? k_store_finalize<4> : k_store_finalize<1>, grid_for(n, many ? 1024 : 256), 256, s,
+                     (const pk_entry *)ctx->table, n, key_off, R, result, slot_out, ctx->counter_dev);
+}
+
 cudaError_t pk_launch_store(const pk_ctx *ctx, unsigned long long epoch, const uint8_t *keys,
                             const uint32_t *slots, uint64_t n, const int64_t *key_off,
                             const int32_t *hit_chunks, uint32_t R, int32_t *result, uint32_t *slot_out,
@@ -1372,8 +1411,7 @@ cudaError_t pk_launch_store(const pk_ctx *ctx, unsigned long long epoch, const u
                       ctx->counter_dev, epoch, ctx->stamps, keys, slots, n, key_off, hit_chunks, R, result, slot_out, status);
     }
     if (e == cudaSuccess)
-        e = pk_launch(k_store_finalize, grid_for(n, 256), 256, s, (const pk_entry *)ctx->table, n, key_off, R, result,
-                      slot_out, ctx->counter_dev);
+        e = launch_finalize(ctx, n, key_off, R, result, slot_out, s);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1411,8 +1449,7 @@ cudaError_t pk_launch_lookup_store(const pk_ctx *ctx, unsigned long long epoch, 
                           (const uint32_t *)slots, hit_chunks, result, slot_out, status);
     }
     if (e == cudaSuccess && key_capacity)
-        e = pk_launch(k_store_finalize, grid_for(key_capacity, 256), 256, s, (const pk_entry *)ctx->table,
-                      key_capacity, key_off, R, result, slot_out, ctx->counter_dev);
+        e = launch_finalize(ctx, key_capacity, key_off, R, result, slot_out, s);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
