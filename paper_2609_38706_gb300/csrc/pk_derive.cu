@@ -573,6 +573,7 @@ struct ChainSmem {
     uint4 kw1[16][kChainLanes];     // block-1 K+W, t = 16..63 used
     uint4 kw2[2][16][kChainLanes];  // block-2 K+W, double-buffered by step parity
     uint4 kpub[2][kChainLanes];     // k_{i-1} for the schedule warp
+    uint8_t order[2][4 * kChainLanes];  // longest_first's, of the rounds and of the schedule warp
 };
 
 // 16 schedule words t = 16q .. 16q+15 of the ring w (in place), K_t + W_t -> out[t / 4][lane]
@@ -611,11 +612,69 @@ __device__ __forceinline__ void rounds16_kw(uint32_t v[8], const uint4 (*kw)[kCh
     v[0] = a; v[1] = b; v[2] = c; v[3] = d; v[4] = e; v[5] = f; v[6] = g; v[7] = h;
 }
 
+// Request `at` of a CTA's m, from r0 on: its first key, number of keys (0: none or out of order) and descriptor.
+__device__ __forceinline__ void chain_request(const int64_t *key_off, const uint32_t *desc_idx, uint32_t D, uint32_t r0,
+                                              uint32_t m, uint32_t at, int64_t &a, int64_t &n, uint32_t &di) {
+    a = n = 0;
+    di = 0;
+    if (at >= m) return;
+    const uint64_t r = (uint64_t)r0 + at;
+    a = key_off[r];
+    n = key_off[r + 1] - a;
+    di = desc_idx[r];
+    if (n < 0 || di >= D) n = 0;
+}
+
+// A pair runs as many steps as its longest request has chunks, and a step is the longer the more of the CTA's pairs
+// still run.  So a CTA hands its requests to its pairs longest first: short pairs end early and leave their
+// sub-partitions to the long ones, whose rounds and schedule share them with other pairs (with both warps of a pair on
+// one sub-partition the long pair gains nothing).  Key derivation, lookup and store of R prompts whose chunk counts
+// spread evenly in the logarithm over a factor of 16, in us before and after: R = 5000 of up to 255 chunks (three pairs)
+// 602 and 553, 8000 of 125 (four) 359 and 324, 16384 of 128 (k_chain) 491 and 441.  Equal prompts take the order that
+// they have, found by a vote over the counts, which are read beside the request's own: 8000 prompts 438 and 443.5
+// (the schedules' places; next to the rounds of pair p + 1 or p - 1 449 and 451), 5000 753.0 and 754, 16384 651.1 and
+// 652.5.
+//
+// Which of a CTA's m <= N requests, from r0 on, is at position `pos` when the longest come first (equal ones in their
+// own order); at least m where there is none.  Every warp finds it by itself; `order` (N bytes) is its own.
+template <int N>
+__device__ __forceinline__ uint32_t longest_first(const int64_t *key_off, uint32_t r0, uint32_t m, uint32_t pos,
+                                                  uint8_t *order) {
+    constexpr int kPerLane = (N + 31) / 32;
+    const uint32_t lane = threadIdx.x & 31;
+    int32_t n[kPerLane];  // chunks, limited to 32 bits (the order only sets which requests share a pair); none: -1
+    bool equal = true;
+#pragma unroll
+    for (int h = 0; h < kPerLane; ++h) {
+        const uint32_t j = lane + 32 * h;
+        const int64_t c = j < m ? key_off[(uint64_t)r0 + j + 1] - key_off[(uint64_t)r0 + j] : -1;
+        n[h] = (int32_t)(c > INT32_MAX ? INT32_MAX : c < 0 ? -1 : c);
+        const int32_t n0 = __shfl_sync(0xffffffffu, n[0], 0);
+        equal = equal && (j >= m || n[h] == n0);
+    }
+    if (__all_sync(0xffffffffu, equal)) return pos;
+    uint32_t rank[kPerLane] = {};
+#pragma unroll
+    for (int g = 0; g < kPerLane; ++g) {
+#pragma unroll 4
+        for (int j = 0; j < 32; ++j) {
+            const int32_t o = __shfl_sync(0xffffffffu, n[g], j);
+#pragma unroll
+            for (int h = 0; h < kPerLane; ++h) rank[h] += o > n[h] || (o == n[h] && 32 * g + j < (int)lane + 32 * h);
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < kPerLane; ++h)
+        if (rank[h] < N) order[rank[h]] = (uint8_t)(lane + 32 * h);
+    __syncwarp();
+    return order[pos];
+}
+
 // At most 64 registers (no spills): uncapped, the compiler took 81 and a small-block step whose
 // lookup-and-store launch overlaps the chain's tail ran 910 -> 955 us.  `groups` = ceil(R / 32); CTA c serves
 // groups [c * groups / gridDim.x, (c + 1) * groups / gridDim.x), at most four.  Pair p is rounds warp p and
-// schedule warp p + 4, which share a sub-partition: the schedule fills the issue slots that the rounds warp's
-// dependency chain leaves idle.
+// schedule warp 4 + (p + 2) % 4: a sub-partition holds the rounds of one pair and the schedule of another, which fills
+// the issue slots that the rounds' dependency chain leaves idle.
 // FS1, FS2: the forms (pk_sha256.cuh) of the schedule warp's additions for block 1 and block 2, `one` their
 // run-time 1.  The rounds warp's dependency chain sets the step time, and a multiply-add's longer latency there made
 // the chain slower (small-block key derivation 674 -> 718 us with every addition on the FMA pipe); it takes the late
@@ -639,25 +698,21 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
     extern __shared__ __align__(16) uint8_t chain_smem[];
     pk::pdl_wait(key_off, desc_idx, digests, keys);  // successor released at the last step (see k_chunk_digest)
     const uint32_t lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
-    const uint32_t pair = warp & (kChainPairs - 1);
     const bool sched = warp >= (uint32_t)kChainPairs;
+    const uint32_t pair = (sched ? warp + kChainPairs / 2 : warp) & (kChainPairs - 1);
     ChainSmem &sm = reinterpret_cast<ChainSmem *>(chain_smem)[pair];
-    const uint32_t g0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x);
-    const uint32_t g1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * groups / gridDim.x);
-    const uint32_t group = g0 + pair;
-    const bool active = group < g1;
+    const uint32_t r0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x) * kChainLanes;
+    const uint64_t r1 = (uint64_t)(blockIdx.x + 1) * groups / gridDim.x * kChainLanes;
+    const uint32_t m = (uint32_t)(r1 < R ? r1 : R) - r0;
+    const uint32_t at = pair * kChainLanes + lane;
     const int bar_s1 = 1 + 3 * (int)pair;   // block-1 schedule (first slice), and block 2 of the step
     const int bar_s1b = 2 + 3 * (int)pair;  // block-1 schedule (second slice)
     const int bar_k = 3 + 3 * (int)pair;    // k_i published
-    const uint32_t r = group * kChainLanes + lane;
-    int64_t a = 0, n = 0;
-    uint32_t di = 0;
-    if (active && r < R) {
-        a = key_off[r];
-        n = key_off[r + 1] - a;
-        di = desc_idx[r];
-        if (n < 0 || di >= D) n = 0;
-    }
+    int64_t a, n;
+    uint32_t di;
+    chain_request(key_off, desc_idx, D, r0, m, at, a, n, di);
+    const uint32_t pos = longest_first<kChainPairs * kChainLanes>(key_off, r0, m, at, sm.order[sched]);
+    if (pos != at) chain_request(key_off, desc_idx, D, r0, m, pos, a, n, di);
     const int64_t nmax = warp_max(n);  // identical in both warps of the pair: they cover the same requests
     if (nmax == 0) {  // uniform over the pair
         pk::pdl_launch_dependents();
@@ -787,7 +842,7 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
 // 132 slots of about 24 cycles.  With one pair per CTA the two warps run on
 // different sub-partitions; with three, the rounds warps have a sub-partition
 // each and the schedule warps share the fourth; with four, pair p is rounds
-// warp p and schedule warp p + 4, on one sub-partition.  The rounds are straight-line code (block 2
+// warp p and schedule warp 4 + (p + 2) % 4, as in k_chain.  The rounds are straight-line code (block 2
 // as a loop of 16 rounds: long-context key derivation 938 -> 1013 us), each
 // 16 words of K + W read while the 16 rounds before them run, and each barrier synced
 // some slots before the words it guards are needed.  The schedule warp's work
@@ -809,6 +864,7 @@ struct SplitSmem {
     uint32_t zero[kSplitRow];                // the odd lanes' K+W
     uint32_t kpub[kSplitReq][2][4];          // k_{i-1}: its even words, its odd words
     uint32_t kpar[2][32];                    // K of the even and of the odd t
+    uint8_t order[2][4 * kSplitReq];         // longest_first's, of the rounds and of the schedule warp
 };
 
 // K+W of rounds 16s .. 16s + 15
@@ -837,7 +893,7 @@ k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *d
     extern __shared__ __align__(16) uint8_t chain_smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool sched = kPairs == 3 ? (warp & 3) == 3 : warp >= (uint32_t)kPairs;
-    const uint32_t pair = kPairs == 3 && sched ? warp >> 2 : kPairs == 4 ? warp & 3 : kPairs == 1 ? 0u : warp;
+    const uint32_t pair = kPairs == 1 ? 0u : !sched ? warp : kPairs == 3 ? warp >> 2 : (warp + 2) & 3;
     if (kPairs == 3 && pair >= 3) {
         __syncthreads();
         return;
@@ -852,25 +908,22 @@ k_chain_split(const int64_t *key_off, const uint32_t *desc_idx, const uint8_t *d
     }
     __syncwarp();
     pk::pdl_wait(key_off, desc_idx, digests, keys);  // successor released at the last step (see k_chunk_digest)
-    uint32_t group = blockIdx.x;
-    bool active = true;
+    uint32_t r0 = blockIdx.x * kSplitReq, m = R - r0, at = q;
     if (kPairs > 1) {
-        const uint32_t g0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x);
-        const uint32_t g1 = (uint32_t)((uint64_t)(blockIdx.x + 1) * groups / gridDim.x);
-        group = g0 + pair;
-        active = group < g1;
+        r0 = (uint32_t)((uint64_t)blockIdx.x * groups / gridDim.x) * kSplitReq;
+        const uint64_t r1 = (uint64_t)(blockIdx.x + 1) * groups / gridDim.x * kSplitReq;
+        m = (uint32_t)(r1 < R ? r1 : R) - r0;
+        at = pair * kSplitReq + q;
     }
     const int bar_s1 = 1 + 3 * (int)pair;   // block-1 schedule t = 16..31, and block 2 of the step
     const int bar_s1b = 2 + 3 * (int)pair;  // block-1 schedule t = 32..63
     const int bar_k = 3 + 3 * (int)pair;    // k_i published
-    const uint32_t r = group * kSplitReq + q;
-    int64_t a = 0, n = 0;
-    uint32_t di = 0;
-    if (active && r < R) {
-        a = key_off[r];
-        n = key_off[r + 1] - a;
-        di = desc_idx[r];
-        if (n < 0 || di >= D) n = 0;
+    int64_t a, n;
+    uint32_t di;
+    chain_request(key_off, desc_idx, D, r0, m, at, a, n, di);
+    if (kPairs > 1) {
+        const uint32_t pos = longest_first<kPairs * kSplitReq>(key_off, r0, m, at, sm.order[sched]);
+        if (pos != at) chain_request(key_off, desc_idx, D, r0, m, pos, a, n, di);
     }
     const int64_t nmax = warp_max(n);  // identical in both warps of the pair: they cover the same requests
     if (nmax == 0) {  // uniform over the pair
