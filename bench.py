@@ -56,8 +56,9 @@ def load_peaks():
     return {"hbm_gbs": 6800.0, "sm_max_mhz": 2070.0, "source": "fallback"}
 
 
-DERIVE_SOURCES = ("paper_2609_38706_gb300/csrc/pk_derive.cu", "paper_2609_38706_gb300/csrc/pk_sha256.cuh",
-                  "paper_2609_38706_gb300/csrc/pk_device.cuh", "paper_2609_38706_gb300/csrc/pk_internal.h")
+DERIVE_SOURCES = ("paper_2609_38706_gb300/csrc/pk_derive.cu", "paper_2609_38706_gb300/csrc/pk_pair.cuh",
+                  "paper_2609_38706_gb300/csrc/pk_sha256.cuh", "paper_2609_38706_gb300/csrc/pk_device.cuh",
+                  "paper_2609_38706_gb300/csrc/pk_internal.h")
 
 
 def derive_traffic(workload: str):

@@ -7,10 +7,11 @@
 //
 // SHA-256 is plain 32-bit integer work: funnel-shift rotates, 3-input logic
 // and 3-input adds, no tensor cores.  The chunk digests are fully parallel
-// (one thread per chunk, message words in registers, 128-bit token loads when
-// the chunk start is 16-byte aligned); the chain is serial per request (one
-// thread per request).  The chunk digests are staged in the output key buffer
-// and overwritten in place by the chain, so derivation needs no scratch memory.
+// (one thread per chunk with the message words in registers, or, when there
+// are few, two lanes of a pair of warps); the chain is serial per request (one
+// or two lanes of a pair of warps).  The chunk digests are staged in the
+// output key buffer and overwritten in place by the chain, so derivation needs
+// no scratch memory.
 #include <cuda_runtime.h>
 
 #include <mutex>
