@@ -39,7 +39,7 @@
 // (gather 37, threshold 5, bitmap and slots 17, compaction 26), against
 // compacting stamps and slots into a list, selecting over it in 5 passes and
 // two more passes for the slots and the bitmap, with one CTA per SM.
-// 2^14 entries, 512 of 5,120 evicted: 54 -> 18 us.
+// 2^14 entries, 512 of 5,120 evicted: 54 -> 18 us (before the parts of k_evict).
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -316,10 +316,20 @@ __device__ __noinline__ void compact_planned(pk_entry *table, unsigned long long
     }
 }
 
+// kParts: 2^parts_log2 threads share a bitmap word in the compaction, each for the clusters that start in its part.  A
+// thread's moves follow one another, loads and stores in turn, so it pays where the grid has threads to spare.
+// The call between two events, without and with parts, in us: 2^20 entries, 600,000 stored, 60,000 evicted 106 and 91 (2
+// parts); 2^18, 64,000 and 16,000, 50 and 45 (8); 2^16, 12,000 and 3,000, 32 and 26; 2^14, 4,800 and 800, 29 and 22;
+// 2^14, 12,000 and 3,000 (long clusters) 293 and 219.  A step of 64 requests under a budget with 512 evictions (2^14):
+// 77.5 and 71.5.  2^21 entries with two parts: 200,000 evicted of 800,000 91 and 86, but 100,000 of 600,000 68 and 72.
+// A table that uses most of the grid takes the other form, which is the code without parts (with them 2^22 entries,
+// one part per word, churn of 262,144 keys 173.0 -> 177.5 us).
+template <bool kParts>
 __global__ void __launch_bounds__(kEvThreads, kEvBlocks)
 k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned long long *counter, uint64_t budget,
         uint64_t keep, unsigned long long epoch, EvictHeader *h, uint32_t *bitmap, uint32_t *evbm, uint8_t *dist,
-        uint32_t *evicted, uint64_t evicted_cap, unsigned long long *n_evicted_out, int32_t *status, BarrierBound bb) {
+        uint32_t *evicted, uint64_t evicted_cap, unsigned long long *n_evicted_out, int32_t *status, BarrierBound bb,
+        uint32_t parts_log2) {
     __shared__ unsigned int sh_hist[256];
     __shared__ unsigned long long sh_sel[3];
     __shared__ unsigned long long sh_count[2];
@@ -525,18 +535,26 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
     if (!grid_sync(h, barrier++, status, bb)) return;
     if (gtid == 0 && n_evicted_out) *n_evicted_out = __ldcg(&h->n_evicted);
     if (n > keep) {
-        // 4b. compaction: one thread per bitmap word, for the clusters that start in it and lose an entry.  Clusters
+        // 4b. compaction: one thread per bitmap word or part of one, for the clusters that start in it and lose an entry.  Clusters
         // that end within the 64 positions of the word and the next one are planned in registers
         // from the occupancy, evicted and distance bytes; the word's moves then go out four loads
         // at a time.  Longer clusters take compact_planned (the same plan, 32 positions at a time),
         // tables below 64 entries and clusters beyond kPlanMax compact_walk.
         const uint64_t n_words = (capacity + 31) / 32;
-        // 32 words per warp, the warps in turn over the CTAs (a small table's words spread over the SMs)
-        for (uint64_t w = ((uint64_t)(tid >> 5) * gridDim.x + blockIdx.x) * 32 + lane; w < n_words; w += nthreads) {
+        // 32 neighbouring words, or parts of words (kParts), per warp, the warps in turn over the CTAs (a small table's
+        // words spread over the SMs)
+        const uint64_t x = ((uint64_t)(tid >> 5) * gridDim.x + blockIdx.x) * 32 + lane;
+        const uint32_t log2 = kParts ? parts_log2 : 0;
+        const uint32_t part = (0xffffffffu >> (32u - (32u >> log2))) << (((uint32_t)x & ((1u << log2) - 1u)) << (5 - log2));
+        for (uint64_t w = x >> log2; w < n_words; w += nthreads) {
             const uint32_t occ_lo = __ldcg(bitmap + w);
             if (!occ_lo) continue;
             const uint32_t before = bit(bitmap, (w * 32 + mask) & mask);  // the position before bit 0
             uint32_t starts = occ_lo & ~((occ_lo << 1) | before);
+            if (kParts) {
+                starts &= part;
+                if (!starts) continue;
+            }
             if (capacity < 64) {
                 while (starts) {
                     const uint32_t b = __ffs(starts) - 1;
@@ -641,17 +659,19 @@ uint64_t pk_evict_scratch_bytes_impl(uint64_t capacity) {
     return kHeaderBytes + 2 * bitmap_bytes(capacity) + 8 * capacity + 4 * capacity + ((capacity + 255) & ~255ull);
 }
 
-// Resident CTAs of k_evict on a device (SMs x CTAs per SM), computed once per device.
+// Resident CTAs of k_evict on a device, in either form (SMs x CTAs per SM), computed once per device.
 static cudaError_t evict_resident(int dev, uint64_t *out) {
     static std::mutex mu;
     static uint64_t cache[256] = {};
     if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (!cache[dev]) {
-        int sms = 0, per_sm = 0;
+        int sms = 0, per_sm = 0, with_parts = 0;
         cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_evict, kEvThreads, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_evict<false>, kEvThreads, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&with_parts, k_evict<true>, kEvThreads, 0);
         if (e != cudaSuccess) return e;
+        if (with_parts < per_sm) per_sm = with_parts;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
         cache[dev] = (uint64_t)sms * per_sm;
     }
@@ -689,7 +709,12 @@ cudaError_t pk_launch_evict(const pk_ctx *ctx, uint64_t budget, uint64_t keep, v
     cfg.numAttrs = 1;
     const BarrierBound bb{spin_limit == 0 || spin_limit > kSpinLimit ? kSpinLimit : spin_limit,
                           withhold_first_cta ? 0u : 0xffffffffu};
-    e = cudaLaunchKernelEx(&cfg, k_evict, ctx->table, ctx->stamps, ctx->capacity, ctx->counter_dev, budget, keep,
-                           ctx->epoch, h, bitmap, evbm, dist, evicted, evicted_cap, n_evicted, status, bb);
+    // At least half of the threads stay without a part, so a thread has one at most.
+    const uint64_t n_words = (ctx->capacity + 31) / 32, threads = (uint64_t)grid * kEvThreads;
+    uint32_t parts_log2 = 0;
+    while (parts_log2 < 3 && n_words << (parts_log2 + 2) <= threads) ++parts_log2;
+    e = cudaLaunchKernelEx(&cfg, parts_log2 ? k_evict<true> : k_evict<false>, ctx->table, ctx->stamps, ctx->capacity,
+                           ctx->counter_dev, budget, keep, ctx->epoch, h, bitmap, evbm, dist, evicted, evicted_cap,
+                           n_evicted, status, bb, parts_log2);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
