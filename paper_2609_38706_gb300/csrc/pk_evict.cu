@@ -318,10 +318,10 @@ __device__ __noinline__ void compact_planned(pk_entry *table, unsigned long long
 
 // kParts: 2^parts_log2 threads share a bitmap word in the compaction, each for the clusters that start in its part.  A
 // thread's moves follow one another, loads and stores in turn, so it pays where the grid has threads to spare.
-// The call between two events, without and with parts, in us: 2^20 entries, 600,000 stored, 60,000 evicted 106 and 91 (2
+// The call between two events, without and with parts, in us: 2^20 entries, 600,000 kept, 60,000 evicted 106 and 91 (2
 // parts); 2^18, 64,000 and 16,000, 50 and 45 (8); 2^16, 12,000 and 3,000, 32 and 26; 2^14, 4,800 and 800, 29 and 22;
 // 2^14, 12,000 and 3,000 (long clusters) 293 and 219.  A step of 64 requests under a budget with 512 evictions (2^14):
-// 77.5 and 71.5.  2^21 entries with two parts: 200,000 evicted of 800,000 91 and 86, but 100,000 of 600,000 68 and 72.
+// 77.5 and 71.5.  2^21 entries with two parts: 200,000 evicted of 1,000,000 91 and 86, but 100,000 of 700,000 68 and 72.
 // A table that uses most of the grid takes the other form, which is the code without parts (with them 2^22 entries,
 // one part per word, churn of 262,144 keys 173.0 -> 177.5 us).
 template <bool kParts>
