@@ -1169,20 +1169,27 @@ k_store_finalize(const pk_entry *table, uint64_t n, const int64_t *key_off, uint
         res[u] = e < n ? result[e] : PK_STORE_SKIPPED;
     }
     if (!any_new && e0 + blockDim.x * (kItems - 1) < total) return;
+    // No claim kernel writes an entry past the batch: its result is whatever the caller's buffer held, PENDING
+    // (the bits of the float 2.0) among it, and its slot_out no position.
     uint32_t pos[kItems];
+    bool pending[kItems];
 #pragma unroll
-    for (uint32_t u = 0; u < kItems; ++u) pos[u] = any_new && res[u] == PK_STORE_PENDING ? slot_out[e0 + u * blockDim.x] : 0u;
+    for (uint32_t u = 0; u < kItems; ++u) {
+        const uint64_t e = e0 + u * blockDim.x;
+        pending[u] = any_new && e < total && res[u] == PK_STORE_PENDING;
+        pos[u] = pending[u] ? slot_out[e] : 0u;
+    }
     unsigned long long w[kItems];
 #pragma unroll
     for (uint32_t u = 0; u < kItems; ++u)
-        w[u] = any_new && res[u] == PK_STORE_PENDING ? *reinterpret_cast<const unsigned long long *>(&table[pos[u]].slot) : 0ull;
+        w[u] = pending[u] ? *reinterpret_cast<const unsigned long long *>(&table[pos[u]].slot) : 0ull;
 #pragma unroll
     for (uint32_t u = 0; u < kItems; ++u) {
         const uint64_t e = e0 + u * blockDim.x;
         if (e >= total && e < n) {
             result[e] = PK_STORE_SKIPPED;
             slot_out[e] = PK_NO_SLOT;
-        } else if (any_new && res[u] == PK_STORE_PENDING) {
+        } else if (pending[u]) {
             result[e] = ~(uint32_t)(w[u] >> 32) == (uint32_t)e ? PK_STORE_INSERTED : PK_STORE_PRESENT;
             slot_out[e] = (uint32_t)w[u];
         }
