@@ -25,6 +25,13 @@ namespace {
 
 using pk::set_status;
 
+// A digest to a 16-byte aligned 32-byte slot.
+__device__ __forceinline__ void store_digest(uint8_t *dst, const uint32_t st[8]) {
+    uint4 *q = reinterpret_cast<uint4 *>(dst);
+    q[0] = make_uint4(pk::bswap32(st[0]), pk::bswap32(st[1]), pk::bswap32(st[2]), pk::bswap32(st[3]));
+    q[1] = make_uint4(pk::bswap32(st[4]), pk::bswap32(st[5]), pk::bswap32(st[6]), pk::bswap32(st[7]));
+}
+
 // ---------------------------------------------------------------------------
 // Descriptor digests: one warp per descriptor.  The warp copies the encoding
 // into shared memory with coalesced byte loads (32 bytes per round trip), then
@@ -64,7 +71,9 @@ __device__ __forceinline__ void hash_descriptor_bytes(uint8_t *stage, const uint
     if (lane == 0) pk::sha256_bytes(staged ? stage : enc + a, (uint64_t)len, digests + 32ull * j);
 }
 
-// stage: kDescStage bytes, 16-byte aligned; sK: the round constants.
+// stage: kDescStage bytes, 16-byte aligned; sK: the round constants; kAligned: digests is 16-byte aligned (else it
+// may lie anywhere).
+template <bool kAligned>
 __device__ __forceinline__ void hash_descriptor(uint8_t *stage, const uint32_t *sK, const uint8_t *enc, uint64_t enc_bytes,
                                                 const int64_t *enc_off, uint32_t j,
                                                 uint8_t *digests, int32_t *status) {
@@ -98,9 +107,13 @@ __device__ __forceinline__ void hash_descriptor(uint8_t *stage, const uint32_t *
             for (int t = 0; t < 16; ++t) w[t] = pk::bswap32(words[16 * blk + t]);
             pk::compress_rolled(st, w, sK);
         }
-        uint4 *q = reinterpret_cast<uint4 *>(digests + 32ull * j);
-        q[0] = make_uint4(pk::bswap32(st[0]), pk::bswap32(st[1]), pk::bswap32(st[2]), pk::bswap32(st[3]));
-        q[1] = make_uint4(pk::bswap32(st[4]), pk::bswap32(st[5]), pk::bswap32(st[6]), pk::bswap32(st[7]));
+        uint8_t *d = digests + 32ull * j;
+        if (kAligned || (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
+            store_digest(d, st);
+        } else {
+#pragma unroll
+            for (int t = 0; t < 32; ++t) d[t] = (uint8_t)(st[t / 4] >> (24 - 8 * (t % 4)));
+        }
     }
 }
 
@@ -115,7 +128,7 @@ k_digest_descriptors(const uint8_t *enc, uint64_t enc_bytes, const int64_t *enc_
     pk::pdl_wait(enc, enc_off, digests, status);
     const uint32_t warp = threadIdx.x >> 5;
     const uint32_t j = blockIdx.x * kDescWarps + warp;
-    if (j < D) hash_descriptor(stage[warp], sK, enc, enc_bytes, enc_off, j, digests, status);
+    if (j < D) hash_descriptor<false>(stage[warp], sK, enc, enc_bytes, enc_off, j, digests, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -241,12 +254,6 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
         key_off[0] = 0;
         if (bad) set_status(status, PK_ERR_ARG);
     }
-}
-
-__device__ __forceinline__ void store_digest(uint8_t *dst, const uint32_t st[8]) {
-    uint4 *q = reinterpret_cast<uint4 *>(dst);
-    q[0] = make_uint4(pk::bswap32(st[0]), pk::bswap32(st[1]), pk::bswap32(st[2]), pk::bswap32(st[3]));
-    q[1] = make_uint4(pk::bswap32(st[4]), pk::bswap32(st[5]), pk::bswap32(st[6]), pk::bswap32(st[7]));
 }
 
 // 16 message words of one 64-byte block of int32 tokens (little-endian bytes,
@@ -490,7 +497,7 @@ k_chunk_digest_pairs(const int32_t *tokens, const int64_t *tok_off, const int64_
         const uint32_t warp = threadIdx.x >> 5;
         const uint32_t j = blockIdx.x * kDescWarps + warp;
         uint8_t *stage = reinterpret_cast<uint8_t *>(sm.ring) + warp * kDescStage;
-        if (warp < kDescWarps && j < dw.D) hash_descriptor(stage, sK, enc, dw.enc_bytes, enc_off, j, digests, dstatus);
+        if (warp < kDescWarps && j < dw.D) hash_descriptor<true>(stage, sK, enc, dw.enc_bytes, enc_off, j, digests, dstatus);
         pk::pdl_launch_dependents();
         return;
     }
