@@ -30,7 +30,7 @@ struct pk_ctx {
     unsigned long long *counter_dev;  // [0] entries in the table; [1] requests handed out by a lookup-and-store;
                                       // [2] entries deferred in a store call; [3], [4] keys its claims and its
                                       // admission pass claimed (folded into [0] by its finalize kernel); [5] CTAs
-                                      // of its claim kernel done; [6] whether the call claimed a key
+                                      // of its claim kernel done; [6] whether an entry of the call may be PENDING
     unsigned long long epoch;         // last store call number
     unsigned long long *stamps;       // budget mode: last-use stamp per entry (pk_attach_stamps), else NULL
     uint32_t pad_kw[64];              // K_t + W_t of a chunk's final (padding-only) block, C % 16 == 0

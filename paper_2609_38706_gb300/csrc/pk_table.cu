@@ -385,10 +385,11 @@ k_first_miss(const int64_t *key_off, uint32_t R, uint64_t key_capacity,
 // Context counter words: [0] entries in the table at the start of the call
 // (constant while its claim kernel runs, so that every warp takes the same
 // mode), [1] requests handed out by a work-taking lookup-and-store, [2]
-// entries deferred in this call, [3] keys its claims claimed, [4] keys its
-// admission pass claimed, [5] CTAs of the claim kernel done (reset by the
-// last), [6] whether the call claimed a key (set by the last); the finalize
-// kernel adds [3] and [4] to [0] and clears [2..4].
+// entries deferred in this call, [3] keys its claims claimed (low half) and
+// CTAs with an entry that ended PENDING (high half), [4] keys
+// its admission pass claimed, [5] CTAs of the claim kernel done (reset by the
+// last), [6] whether an entry of the call may be PENDING (set by the last); the
+// finalize kernel adds the claims of [3] and [4] to [0] and clears [2..4].
 // ---------------------------------------------------------------------------
 enum Examine { kAdvance, kDone, kClaimedHere };
 enum ClaimMode : uint32_t {
@@ -642,17 +643,29 @@ __device__ __forceinline__ bool in_store_range(const int64_t *key_off, const int
     return in_range;
 }
 
-// Adds the warp's claims and deferred entries to the block totals, then the
-// block totals to counter[3] (claims) and counter[2] (deferred): one atomic
-// per block and word (same-address atomics serialise in L2).
+// A lane's count of DEFERRED entries, with kPendingSeen once one was PENDING.
+constexpr uint32_t kPendingSeen = 0x80000000u;
+
+__device__ __forceinline__ void count_state(int32_t res, uint32_t &deferred) {
+    if (res < PK_STORE_PENDING) return;
+    if (res == PK_STORE_DEFERRED) ++deferred;
+    else deferred |= kPendingSeen;
+}
+
+// Adds the warp's claims and deferred entries (count_state's) to the block
+// totals, then the block totals to counter[3] (claims, and 2^32 when an entry
+// of the block is PENDING) and counter[2] (deferred): one atomic per block and
+// word (same-address atomics serialise in L2).
 __device__ __forceinline__ void count_claims(unsigned long long *block_sums, uint32_t claims, uint32_t deferred,
                                              unsigned long long *counter) {
     const uint32_t w = __reduce_add_sync(kFull, claims);
-    const uint32_t d = __reduce_add_sync(kFull, deferred);
-    if ((threadIdx.x & 31) == 0 && w) atomicAdd_block(block_sums, (unsigned long long)w);
+    const uint32_t d = __reduce_add_sync(kFull, deferred & ~kPendingSeen);
+    const unsigned long long lw = (__any_sync(kFull, deferred & kPendingSeen) ? 1ull << 32 : 0ull) | w;
+    if ((threadIdx.x & 31) == 0 && lw) atomicAdd_block(block_sums, lw);
     if ((threadIdx.x & 31) == 0 && d) atomicAdd_block(block_sums + 1, (unsigned long long)d);
     __syncthreads();
-    if (threadIdx.x == 0 && block_sums[0]) atomicAdd(counter + 3, block_sums[0]);
+    if (threadIdx.x == 0 && block_sums[0])  // (a block's warps may each have set the high half)
+        atomicAdd(counter + 3, (block_sums[0] >> 32 ? 1ull << 32 : 0ull) | (uint32_t)block_sums[0]);
     if (threadIdx.x == 0 && block_sums[1]) atomicAdd(counter + 2, block_sums[1]);
 }
 
@@ -674,8 +687,8 @@ __device__ __forceinline__ void admit_write(uint64_t e, int32_t res, uint32_t ou
 
 // Store, admission pass (see the store comment above), run by one CTA: the
 // last CTA of the claim kernel to finish.  The call's entries are [0, n), or
-// [0, min(n, key_off[R])) in range and lookup-and-store mode; counter[0] +
-// counter[3] is the entry count after the claims, counter[2] the number of
+// [0, min(n, key_off[R])) in range and lookup-and-store mode; counter[0] + the
+// claims of counter[3] is the entry count after the claims, counter[2] the number of
 // DEFERRED entries; keys claimed here are added to counter[4].  Within the
 // call the entry count can only reach capacity - 1: the claim kernel claims
 // only when the whole call fits, and here at most `room` keys are claimed.
@@ -689,7 +702,7 @@ __device__ __noinline__ void store_admit(pk_entry *table, uint64_t mask, uint32_
     __shared__ unsigned long long s_claims;
     const unsigned long long deferred = __ldcg(counter + 2);
     if (deferred == 0) return;  // every key was decided by the claim kernel
-    const unsigned long long count = __ldcg(counter) + __ldcg(counter + 3);
+    const unsigned long long count = __ldcg(counter) + (uint32_t)__ldcg(counter + 3);
     const unsigned long long room = count + 1 < capacity ? capacity - 1 - count : 0ull;
     uint64_t end = n;
     if (key_off) {
@@ -765,15 +778,17 @@ __device__ __noinline__ void store_admit(pk_entry *table, uint64_t mask, uint32_
 
 // End of a claim kernel: the last CTA to finish (every CTA counts itself on
 // counter[5] after a fence) runs the admission pass when the call deferred
-// entries, resets counter[5] for the next call, and sets *any_new (if given) to
-// whether the call claimed a key: without one no entry is PENDING.  Every CTA
-// of the grid must call it.
+// entries, resets counter[5] for the next call, and sets *any_pending (if
+// given): 0 only when no entry of the call is PENDING.  (A claim alone would
+// not tell: replayed from a CUDA graph, a call meets the entries of its own
+// number that it claimed before, and bids on them.)  Every CTA of the grid
+// must call it.
 __device__ __forceinline__ void admit_if_last(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t capacity,
                                               unsigned long long *counter, unsigned long long epoch,
                                               unsigned long long *stamps, const uint8_t *keys, const uint32_t *slots,
                                               uint64_t n, const int64_t *key_off, uint32_t R, int32_t *result,
                                               uint32_t *slot_out, uint32_t *pos_out, int32_t *status,
-                                              unsigned long long *any_new) {
+                                              unsigned long long *any_pending) {
     __shared__ int s_last;
     __threadfence();  // this CTA's results and counts are visible to the GPU before it counts itself
     __syncthreads();
@@ -783,14 +798,10 @@ __device__ __forceinline__ void admit_if_last(pk_entry *table, uint64_t mask, ui
     __threadfence();
     if (threadIdx.x == 0) counter[5] = 0;
     const unsigned long long deferred = __ldcg(counter + 2);
-    unsigned long long claimed = __ldcg(counter + 3);
-    if (deferred) {  // else the claim kernel decided every entry
+    if (threadIdx.x == 0 && any_pending) *any_pending = (deferred | __ldcg(counter + 3)) != 0ull;
+    if (deferred)  // else the claim kernel decided every entry
         store_admit(table, mask, max_probe, capacity, counter, epoch, stamps, keys, slots, n, key_off, R, result,
                     slot_out, pos_out, status);
-        __syncthreads();  // the admission pass has added its claims
-        claimed |= __ldcg(counter + 4);
-    }
-    if (threadIdx.x == 0 && any_new) *any_new = claimed != 0ull;
 }
 
 // List mode, or range mode for few long requests: one warp per 32
@@ -826,7 +837,9 @@ k_store_claim(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t capac
         if (res < 0) set_status(status, res);
     }
     pk::pdl_launch_dependents();
-    count_claims(block_sums, claims, e < n && res == PK_STORE_DEFERRED, counter);
+    uint32_t deferred = 0;
+    count_state(res, deferred);  // (SKIPPED past the entries)
+    count_claims(block_sums, claims, deferred, counter);
     admit_if_last(table, mask, max_probe, capacity, counter, epoch, stamps, keys, slots, n, key_off, R, result, slot_out,
                   slot_out, status, counter + 6);
 }
@@ -909,7 +922,7 @@ k_store_claim_req(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t c
             result[s.e] = res;
             slot_out[s.e] = out;
             if (res < 0) set_status(status, res);
-            deferred += res == PK_STORE_DEFERRED;
+            count_state(res, deferred);
         }
     }
     pk::pdl_launch_dependents();
@@ -996,7 +1009,7 @@ __device__ __forceinline__ void lookup_store_request(const ClaimCtx &c, uint64_t
             slots[e] = lslot;
             result[e] = res;
             slot_out[e] = out;
-            deferred += res == PK_STORE_DEFERRED;
+            count_state(res, deferred);
             if (lslot == PK_NO_SLOT) {
                 first_miss = min(first_miss, (uint32_t)(e - a));
                 if (res < 0) set_status(status, res);
@@ -1095,7 +1108,9 @@ k_lookup_store(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t capa
         if (lslot == PK_NO_SLOT && res < 0) set_status(status, res);
     }
     pk::pdl_launch_dependents();
-    count_claims(block_sums, claims, e < end && res == PK_STORE_DEFERRED, counter);
+    uint32_t deferred = 0;
+    count_state(res, deferred);  // (SKIPPED past the entries)
+    count_claims(block_sums, claims, deferred, counter);
     admit_if_last(table, mask, max_probe, capacity, counter, epoch, stamps, keys, new_slots, key_capacity, key_off, R,
                   result, slot_out, slot_out, status, counter + 6);
 }
@@ -1138,24 +1153,24 @@ k_lookup_store_tail(const int64_t *key_off, uint32_t R, uint64_t key_capacity,
 // final once every claim is in: the lowest claimant is INSERTED, the others
 // PRESENT with its slot.  In range mode, entries past key_off[R] (not keys
 // of this batch) are skipped.  The call's claims are added to the entry
-// count, and its counter words [2..4] cleared.  counter[6] says whether the
-// call claimed a key at all: in a call that did not (every key found) a thread
+// count, and its counter words [2..4] cleared.  counter[6] says whether an
+// entry may be PENDING at all: in a call without (every key found) a thread
 // leaves after its first loads.  kItems entries per thread, their loads in
 // flight together: four for calls of more entries than the SMs hold threads
 // (small-block lookup and store, 2.1 M keys all found: 100.6 us with one, 91.2
 // with four), one below (262,144 inserts: four cost 1.3 us more).
 template <uint32_t kItems>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 6)
 k_store_finalize(const pk_entry *table, uint64_t n, const int64_t *key_off, uint32_t R,
                  int32_t *result, uint32_t *slot_out, unsigned long long *counter) {
     pk::pdl_launch_dependents();
     pk::pdl_wait(table, key_off, result, slot_out, counter);
-    const bool any_new = __ldcg(counter + 6) != 0ull;
+    const bool any_pending = __ldcg(counter + 6) != 0ull;
     const uint64_t total = key_off ? (R > 0 ? (uint64_t)__ldcg(key_off + R) : 0ull) : n;
     const uint64_t e0 = (uint64_t)blockIdx.x * (blockDim.x * kItems) + threadIdx.x;
     if (e0 == 0) {
         const unsigned long long c2 = __ldcg(counter + 2), c3 = __ldcg(counter + 3), c4 = __ldcg(counter + 4);
-        if (c3 | c4) counter[0] += c3 + c4;
+        if (c3 | c4) counter[0] += (uint32_t)c3 + c4;
         if (c2 | c3 | c4) {
             counter[2] = 0;
             counter[3] = 0;
@@ -1168,30 +1183,29 @@ k_store_finalize(const pk_entry *table, uint64_t n, const int64_t *key_off, uint
         const uint64_t e = e0 + u * blockDim.x;
         res[u] = e < n ? result[e] : PK_STORE_SKIPPED;
     }
-    if (!any_new && e0 + blockDim.x * (kItems - 1) < total) return;
+    if (!any_pending && e0 + blockDim.x * (kItems - 1) < total) return;
     // No claim kernel writes an entry past the batch: its result is whatever the caller's buffer held, PENDING
     // (the bits of the float 2.0) among it, and its slot_out no position.
     uint32_t pos[kItems];
-    bool pending[kItems];
 #pragma unroll
     for (uint32_t u = 0; u < kItems; ++u) {
         const uint64_t e = e0 + u * blockDim.x;
-        pending[u] = any_new && e < total && res[u] == PK_STORE_PENDING;
-        pos[u] = pending[u] ? slot_out[e] : 0u;
+        if (!any_pending || e >= total) res[u] = PK_STORE_SKIPPED;
+        pos[u] = res[u] == PK_STORE_PENDING ? slot_out[e] : 0u;
     }
     unsigned long long w[kItems];
 #pragma unroll
     for (uint32_t u = 0; u < kItems; ++u)
-        w[u] = pending[u] ? *reinterpret_cast<const unsigned long long *>(&table[pos[u]].slot) : 0ull;
+        w[u] = res[u] == PK_STORE_PENDING ? *reinterpret_cast<const unsigned long long *>(&table[pos[u]].slot) : 0ull;
 #pragma unroll
     for (uint32_t u = 0; u < kItems; ++u) {
         const uint64_t e = e0 + u * blockDim.x;
-        if (e >= total && e < n) {
-            result[e] = PK_STORE_SKIPPED;
-            slot_out[e] = PK_NO_SLOT;
-        } else if (pending[u]) {
+        if (res[u] == PK_STORE_PENDING) {
             result[e] = ~(uint32_t)(w[u] >> 32) == (uint32_t)e ? PK_STORE_INSERTED : PK_STORE_PRESENT;
             slot_out[e] = (uint32_t)w[u];
+        } else if (e >= total && e < n) {
+            result[e] = PK_STORE_SKIPPED;
+            slot_out[e] = PK_NO_SLOT;
         }
     }
 }
@@ -1243,7 +1257,7 @@ __global__ void k_mark_loaded(pk_entry *table, uint64_t capacity) {
 struct NoallocScratch {
     // [0] entries in the table (set by the scan), [1] largest call number
     // found in the table, [2] entries deferred in this call, [3] keys its
-    // claims claimed, [4] keys its admission pass claimed, [5] CTAs of the
+    // claims claimed (low half), [4] keys its admission pass claimed, [5] CTAs of the
     // claim kernel done: [0] and [2..5] are the words a context's counter
     // holds at the same indices
     unsigned long long word[6];
@@ -1313,7 +1327,9 @@ k_noalloc_claim(pk_entry *table, uint64_t mask, uint32_t max_probe, uint64_t cap
         }
         if (res < 0) set_status(status, res);
     }
-    count_claims(block_sums, claims, e < n && res == PK_STORE_DEFERRED, sc->word);
+    uint32_t deferred = 0;
+    count_state(res, deferred);  // (SKIPPED past the entries)
+    count_claims(block_sums, claims, deferred, sc->word);
     admit_if_last(table, mask, max_probe, capacity, sc->word, epoch, nullptr, keys, slots, n, key_off, R, result,
                   slot_out, sc->pos, status, nullptr);
 }
