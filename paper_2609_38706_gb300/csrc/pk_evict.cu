@@ -18,7 +18,9 @@
 //      the budget (the common step costs one short launch);
 //   2. gather: one bit per entry (occupied), one byte with its distance from
 //      home, the numbers of entries with and without a stamp, the range of
-//      the stamps, and a histogram of their age in store calls;
+//      the stamps, and a histogram of their age in store calls
+//      (an eviction replayed from a CUDA graph has the call number of its
+//      capture: calls after that count as age 0);
 //   3. the threshold v: the age histogram gives the call in which the last
 //      entry to go was used; if every entry of that call and the calls before
 //      it goes, v is known (a store that evicts whole batches, the common
@@ -383,7 +385,7 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
             }
             uint32_t bin = 256;
             if (occ && st[u]) {
-                const unsigned long long age = epoch - (st[u] >> 32);
+                const unsigned long long call = st[u] >> 32, age = call < epoch ? epoch - call : 0ull;
                 bin = by_age && age < 255 ? (uint32_t)age : 255u;
                 ++stamped;
                 lo = st[u] < lo ? st[u] : lo;
@@ -431,9 +433,12 @@ k_evict(pk_entry *table, unsigned long long *stamps, uint64_t capacity, unsigned
             pick_bucket(h->age, true, n - keep - 1 - n0, sh_sel);  // oldest first
             const unsigned long long age = sh_sel[0];
             unsigned long long rank = sh_sel[1], left = sh_sel[2];
-            // the candidates' range [clo, chi]
+            // the candidates' range [clo, chi] (age 0: the call `epoch` and the calls after it)
             unsigned long long clo = age < 255 ? (epoch - age) << 32 : 0ull;
-            unsigned long long chi = age < 255 ? clo | __ldcg(&h->max_index) : by_age ? ((epoch - 254) << 32) - 1 : ~0ull;
+            unsigned long long chi = age == 0 ? smax
+                                     : age < 255 ? clo | __ldcg(&h->max_index)
+                                     : by_age    ? ((epoch - 254) << 32) - 1
+                                                 : ~0ull;
             clo = clo > smin ? clo : smin;
             chi = chi < smax ? chi : smax;
             __syncthreads();

@@ -67,3 +67,37 @@ def test_store_again(log2, mode, R, per):
     status = kt.take_status()
     assert status == (pk.PK_OK if log2 == 12 else pk.PK_ERR_TABLE_FULL)
     kt.close()
+
+
+@pytest.mark.parametrize("calls", [4, 300])  # calls before the capture, 25 keys each
+@pytest.mark.parametrize("keep", [1, 24, 40, 50, 60, 99, 100, 120, 149])
+def test_evict_after_later_calls(keep, calls):
+    """An eviction captured before the last stores: the calls after it are the newest."""
+    rng = np.random.default_rng(keep)
+    n = 25 * (calls + 2)
+    keys, slots = random_keys(rng, n), np.arange(n, dtype=np.uint32)
+    kt, bt = KeyTable(16, 14), O.BudgetTable(1 << 14)
+    kt.attach_stamps()
+
+    def store(a, b):
+        kt.store(keys[a:b], slots[a:b])
+        bt.store(keys[a:b], slots[a:b])
+
+    for c in range(calls):
+        store(25 * c, 25 * c + 25)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ev, n_ev = kt.evict(keep, keep)
+    for c in (calls, calls + 1):
+        store(25 * c, 25 * c + 25)
+    for again in range(2):
+        g.replay()
+        want = bt.evict(keep, keep)
+        torch.cuda.synchronize()
+        kt.check("evict")
+        assert np.array_equal(np.sort(ev[: int(n_ev.item())].cpu().numpy().view(np.uint32)), want)
+        _, got = kt.lookup(torch.from_numpy(keys).cuda(), torch.arange(n + 1, dtype=torch.int64, device="cuda"))
+        assert np.array_equal(got.cpu().numpy().view(np.uint32), bt.table.get(keys))
+        store(0, 25)
+    kt.close()
