@@ -135,16 +135,21 @@ k_digest_descriptors(const uint8_t *enc, uint64_t enc_bytes, const int64_t *enc_
 // Chunk offsets: one block per tile of kScanThreads * kScanItems requests.
 // Each block scans its own tile (kScanItems consecutive requests per thread)
 // and sums the requests of every other tile with independent, coalesced loads:
-// those before it give its first offset, all of them the checks.  That is more
-// loads, but no block waits for another and none walks the tiles one after the
-// other (key derivation of 16,384 prompts of 32 tokens 37.6 -> 29.1 us, of 100,000
-// 171 -> 100 us).  Any invalid request (offsets
-// decreasing, negative or past n_tokens, descriptor index >= D) or a total
-// above key_capacity makes all offsets zero and reports PK_ERR_ARG.
+// those before it give its first offset, all of them the checks.  No block waits
+// for another and none scans the tiles one after the other (key derivation of
+// 16,384 prompts of 32 tokens 37.6 -> 29.1 us, of 100,000 171 -> 100 us), but
+// every block reads every request, so the loads grow with the square of R: above
+// kScanTiles tiles one block walks the tiles instead (k_chunk_offsets_walk).
+// This launch alone, every block reading all | one block, in us, R = 2^17:
+// 43.9 | 138, 2^20: 627 | 1093, 1.48 M: 1319 | 1544, 2^21: 2473 | 2178,
+// 2^23: 38332 | 9082.  Any invalid request (offsets decreasing, negative or
+// past n_tokens, descriptor index >= D) or a total above key_capacity makes all
+// offsets zero and reports PK_ERR_ARG.
 // ---------------------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr uint32_t kScanTile = kScanThreads * kScanItems;
+constexpr uint32_t kScanTiles = 360;  // (1.47 M requests)
 
 // Full chunks of the request [a, b) with descriptor index di; bad is set if it is invalid.
 __device__ __forceinline__ long long request_chunks(int64_t a, int64_t b, uint32_t di, uint64_t n_tokens, uint32_t C,
@@ -157,9 +162,28 @@ __device__ __forceinline__ long long request_chunks(int64_t a, int64_t b, uint32
     return len >> 32 ? (long long)(len / C) : (long long)((uint32_t)len / C);
 }
 
+// The requests r0 .. r0 + kScanItems - 1 of a thread: their offsets and descriptor indices.
+__device__ __forceinline__ void load_requests(const int64_t *tok_off, const uint32_t *desc_idx, uint32_t R, uint64_t r0,
+                                              int64_t to[kScanItems + 1], uint32_t di[kScanItems]) {
+#pragma unroll
+    for (int j = 0; j <= kScanItems; ++j) to[j] = r0 + j <= R ? tok_off[r0 + j] : 0;
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) di[j] = r0 + j < R ? desc_idx[r0 + j] : 0u;
+}
+
 __device__ __forceinline__ long long warp_sum(long long x) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Inclusive sum over the lanes.
+__device__ __forceinline__ long long warp_scan(long long x) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long v = __shfl_up_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) >= o) x += v;
+    }
     return x;
 }
 
@@ -182,10 +206,7 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
     bool bad = false;
     int64_t to[kScanItems + 1];
     uint32_t di[kScanItems];
-#pragma unroll
-    for (int j = 0; j <= kScanItems; ++j) to[j] = r0 + j <= R ? tok_off[r0 + j] : 0;
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) di[j] = r0 + j < R ? desc_idx[r0 + j] : 0u;
+    load_requests(tok_off, desc_idx, R, r0, to, di);
     long long before = 0, after = 0;  // chunks of the tiles before and after this one
     for (uint64_t other = 0; kTiles && other < R; other += kScanTile) {
         if (other == base) continue;
@@ -213,12 +234,7 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
         local += n[j];
     }
     // block exclusive scan of the per-thread sums, and the other tiles' totals
-    long long incl = local;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
+    const long long incl = warp_scan(local);
     if (lane == 31) warp_sums[warp] = incl;
     if (kTiles) {
         before = warp_sum(before);
@@ -230,13 +246,7 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
     }
     bad = __syncthreads_or(bad);
     if (warp == 0) {
-        const long long ws = warp_sums[lane];
-        long long wincl = ws;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long v = __shfl_up_sync(0xffffffffu, wincl, o);
-            if (lane >= o) wincl += v;
-        }
+        const long long ws = warp_sums[lane], wincl = warp_scan(ws);
         const long long first = kTiles ? warp_sum(warp_before[lane]) : 0;
         const long long rest = kTiles ? warp_sum(warp_after[lane]) : 0;
         warp_sums[lane] = first + wincl - ws;
@@ -253,6 +263,61 @@ k_chunk_offsets(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t 
     if (blockIdx.x == 0 && tid == 0) {
         key_off[0] = 0;
         if (bad) set_status(status, PK_ERR_ARG);
+    }
+}
+
+// One block, tile after tile, a running carry linking them and each tile's loads in flight during the scan before it.
+__global__ void __launch_bounds__(kScanThreads)
+k_chunk_offsets_walk(const int64_t *tok_off, uint32_t R, uint64_t n_tokens, uint32_t C,
+                     const uint32_t *desc_idx, uint32_t D, uint64_t key_capacity,
+                     int64_t *key_off, int32_t *status) {
+    __shared__ long long warp_sums[kScanThreads / 32];
+    __shared__ long long tile_total;
+    pk::pdl_wait(tok_off, desc_idx, key_off, status);
+    pk::pdl_launch_dependents();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) key_off[0] = 0;
+    bool bad = false;
+    long long carry = 0;
+    int64_t to[kScanItems + 1], to_next[kScanItems + 1] = {};
+    uint32_t di[kScanItems], di_next[kScanItems] = {};
+    load_requests(tok_off, desc_idx, R, (uint64_t)tid * kScanItems, to, di);
+    for (uint64_t base = 0; base < R; base += kScanTile) {
+        const uint64_t r0 = base + (uint64_t)tid * kScanItems;
+        if (base + kScanTile < R) load_requests(tok_off, desc_idx, R, r0 + kScanTile, to_next, di_next);
+        long long n[kScanItems];
+        long long local = 0;
+#pragma unroll
+        for (int j = 0; j < kScanItems; ++j) {
+            n[j] = r0 + j < R ? request_chunks(to[j], to[j + 1], di[j], n_tokens, C, D, bad) : 0;
+            local += n[j];
+        }
+        const long long incl = warp_scan(local);
+        if (lane == 31) warp_sums[warp] = incl;
+        __syncthreads();
+        if (warp == 0) {
+            const long long ws = warp_sums[lane], wincl = warp_scan(ws);
+            warp_sums[lane] = wincl - ws;
+            if (lane == 31) tile_total = wincl;
+        }
+        __syncthreads();
+        long long run = carry + warp_sums[warp] + incl - local;
+#pragma unroll
+        for (int j = 0; j < kScanItems; ++j) {
+            run += n[j];
+            if (r0 + j < R) key_off[r0 + j + 1] = run;
+        }
+        carry += tile_total;
+        __syncthreads();  // warp_sums and tile_total are written again by the next tile
+#pragma unroll
+        for (int j = 0; j <= kScanItems; ++j) to[j] = to_next[j];
+#pragma unroll
+        for (int j = 0; j < kScanItems; ++j) di[j] = di_next[j];
+    }
+    bad = __syncthreads_or(bad);
+    if (bad || (unsigned long long)carry > key_capacity) {
+        for (uint64_t r = tid; r < R; r += kScanThreads) key_off[r + 1] = 0;
+        if (tid == 0) set_status(status, PK_ERR_ARG);
     }
 }
 
@@ -1178,8 +1243,11 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     static_assert(kDigestBlock / 32 * kDescStage <= (int)sizeof(RingStage) * kStages,
                   "descriptor staging fits in the token ring");
     const uint32_t C = ctx->chunk_tokens;
-    cudaError_t e = pk_launch(R <= kScanTile ? k_chunk_offsets<false> : k_chunk_offsets<true>,
-                              R <= kScanTile ? 1 : grid_for(R, kScanTile), kScanThreads, s, tok_off, R, n_tokens, C,
+    const uint32_t tiles = grid_for(R, kScanTile);
+    cudaError_t e = pk_launch(tiles <= 1             ? k_chunk_offsets<false>
+                              : tiles <= kScanTiles ? k_chunk_offsets<true>
+                                                    : k_chunk_offsets_walk,
+                              tiles > kScanTiles || tiles == 0 ? 1 : tiles, kScanThreads, s, tok_off, R, n_tokens, C,
                               desc_idx, D, key_capacity, key_off, status);
     if (e != cudaSuccess) return e;
     DescWork dw = {enc, enc_bytes, enc_off, D, digests, status, 0};
