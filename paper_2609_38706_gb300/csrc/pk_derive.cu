@@ -1254,7 +1254,8 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     if (enc_off) dw.desc_blocks = grid_for(D, kDigestBlock / 32);
     PadKW pad;
     for (int t = 0; t < 64; ++t) pad.kw[t] = ctx->pad_kw[t];
-    const bool chunks = R > 0 && key_capacity > 0;
+    const uint64_t most = n_tokens / C;  // chunks of the batch at most (the caller's buffers may hold many more)
+    const bool chunks = R > 0 && most > 0;
     const uint32_t one = 1u;
     if (chunks) e = raise_smem_limits();
     if (e != cudaSuccess) return e;
@@ -1266,20 +1267,19 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
     }
     // The multiply-add round form pays once two warps of chunks share an SM sub-partition (two warps 4766 against
     // 5191 cycles per compression each, a lone one 3170 against 2830; long-context key derivation, 1.7 warps per
-    // sub-partition, 870.7 -> 868.1 us).  The chunk count is at most key_capacity; with an unknown SM count the
-    // compiler's form is kept.
-    const uint64_t warps = (key_capacity + 31) / 32;
+    // sub-partition, 870.7 -> 868.1 us).  With an unknown SM count the compiler's form is kept.
+    const uint64_t warps = (most + 31) / 32;
     const bool fma = ctx->sm_count > 0 && warps > 4ull * ctx->sm_count;
-    const unsigned grid = grid_for(key_capacity, kDigestBlock) + dw.desc_blocks;
+    const unsigned grid = grid_for(most, kDigestBlock) + dw.desc_blocks;
     // Few chunks: pairs of warps, at most three per SM, on the SMs that the descriptors and the offsets kernel, still
     // running when this launch comes up, leave free.  Key derivation of N chunks (8 per request), one lane per chunk |
     // pairs, in us: chunks of 256, N = 16: 38.0 | 31.4, 2400: 45.4 | 39.2, 7000: 45.6 | 44.6; chunks of 64: 21.1 |
     // 20.9, 28.0 | 27.5, 28.3 | 28.9; chunks of 16: 19.7 | 17.5, 26.2 | 24.8, 26.7 | 25.3.
     const uint32_t desc_sms = enc_off ? grid_for(D, kDescWarps) : 0;
     const uint32_t work = ctx->sm_count > desc_sms + 1 ? ctx->sm_count - desc_sms - 1 : 0;
-    if (C <= 1u << 30 && key_capacity <= (uint64_t)pk::kPairMsgsPerSm * work) {
+    if (C <= 1u << 30 && most <= (uint64_t)pk::kPairMsgsPerSm * work) {
         dw.desc_blocks = desc_sms;
-        const uint64_t pairs = (key_capacity + pk::kPairMsgs - 1) / pk::kPairMsgs;
+        const uint64_t pairs = (most + pk::kPairMsgs - 1) / pk::kPairMsgs;
         e = pk_launch_smem(k_chunk_digest_pairs, (unsigned)(pairs < work ? pairs : work) + desc_sms, pk::kPairThreads,
                            kOnePerSm, s, tokens, tok_off, (const int64_t *)key_off, R, C, pad, keys, dw, one);
     } else if (fma) {
