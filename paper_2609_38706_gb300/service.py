@@ -83,27 +83,30 @@ class KeyTable:
             raise pk.PKError(v, where)
 
     # -- steps -------------------------------------------------------------
-    def _encode(self, descriptors):
+    def _encode(self, descriptors, tensors):
         """The descriptors' encodings and offsets on the device:
         (buffer, address, bytes, offsets' address, D).  Encoded into one pinned
         buffer and copied in one piece, in the order of the table's stream; a
         caller keeps the buffer until its call is enqueued.  (Two copies from
         pageable memory each waited for the stream, and so for the batch
         before, and each descriptor field became three ctypes objects: a step
-        of 8 prompts under 4 descriptors 250 us, 110 now.)"""
+        of 8 prompts under 4 descriptors 250 us, 110 now.)
+
+        ``tensors``: the call's others, made on the current stream.  A table
+        with a stream of its own takes them there behind the current stream's
+        work so far, and their memory is kept until its work is done.  (The
+        copies from pageable memory wait for the current stream on the host.)"""
         stream = self.stream
-        descriptors = descriptors if isinstance(descriptors, pk.Descriptors) else list(descriptors)
         packed = None
         if (stream is None or isinstance(stream, torch.cuda.Stream)) and isinstance(descriptors, list):
             packed = pk.pack_fields(descriptors)
         if packed is not None:
             fields, _, D = packed
             head, bound = 8 * (D + 1), len(fields) + 28 * D
-            if stream is not None:
-                with torch.cuda.stream(stream):
-                    dev = self._encode_packed(packed, head, bound)
-            else:
+            if stream is None:
                 dev = self._encode_packed(packed, head, bound)
+            else:
+                dev = self._encode_on(stream, packed, head, bound, tensors)
             if dev is not None:
                 at = dev.data_ptr()
                 return dev, at + head if D else None, bound, at, D
@@ -111,6 +114,20 @@ class KeyTable:
         enc_d = _dev(enc if enc.size else np.zeros(1, np.uint8), torch.uint8, self.device)
         off_d = _dev(off, torch.int64, self.device)
         return (enc_d, off_d), enc_d.data_ptr() if enc.size else None, enc.size, off_d.data_ptr(), off.size - 1
+
+    def _encode_on(self, stream, packed, head: int, bound: int, tensors) -> Optional[torch.Tensor]:
+        current = torch.cuda.current_stream(self.device)
+        if stream == current:
+            return self._encode_packed(packed, head, bound)
+        if torch.cuda.is_current_stream_capturing():
+            return None
+        with torch.cuda.stream(stream):
+            dev = self._encode_packed(packed, head, bound)
+        if dev is not None:
+            stream.wait_stream(current)
+            for t in tensors:
+                t.record_stream(stream)
+        return dev
 
     def _encode_packed(self, packed, head: int, bound: int) -> Optional[torch.Tensor]:
         if bound > pk.encode_limit(packed[2]) or torch.cuda.is_current_stream_capturing():
@@ -199,7 +216,8 @@ class KeyTable:
     def derive_lookup_store(self, tokens, tok_off, desc_idx, descriptors, new_slots):
         """The whole hot path in one call (pk_derive_lookup_store): returns
         (digests, key_off, keys, hit, slots, result, slot_out)."""
-        enc, enc_at, enc_bytes, off_at, D = self._encode(descriptors)
+        descriptors = descriptors if isinstance(descriptors, pk.Descriptors) else list(descriptors)
+        D = descriptors.count if isinstance(descriptors, pk.Descriptors) else len(descriptors)
         digests = torch.empty((D, 32), dtype=torch.uint8, device=self.device)
         tokens = _dev(tokens, torch.int32, self.device)
         tok_off = _dev(tok_off, torch.int64, self.device)
@@ -214,6 +232,8 @@ class KeyTable:
         slots = torch.empty(max(cap, 0), dtype=torch.int32, device=self.device)
         result = torch.empty(max(cap, 0), dtype=torch.int32, device=self.device)
         slot_out = torch.empty(max(cap, 0), dtype=torch.int32, device=self.device)
+        enc, enc_at, enc_bytes, off_at, D = self._encode(
+            descriptors, (digests, tokens, tok_off, desc_idx, key_off, keys, new_slots, hit, slots, result, slot_out))
         pk.derive_lookup_store_at(self.ctx, tokens, tok_off, desc_idx, enc_at, enc_bytes, off_at, D, digests, key_off, keys,
                                   new_slots, hit, slots, result, slot_out, self.status, self.stream)
         return digests, key_off, keys, hit, slots, result, slot_out
