@@ -23,29 +23,44 @@ def desc(rng, j, extra):
     return d
 
 
-def step(kt, descriptors):
-    return kt.derive_lookup_store(torch.arange(8, dtype=torch.int32, device="cuda"),
-                                  torch.tensor([0, 4, 8], device="cuda"), torch.zeros(2, dtype=torch.int32, device="cuda"),
-                                  descriptors, torch.arange(2, dtype=torch.int32, device="cuda"))
+def step_inputs():
+    return (torch.arange(8, dtype=torch.int32, device="cuda"), torch.tensor([0, 4, 8], device="cuda"),
+            torch.zeros(2, dtype=torch.int32, device="cuda"), torch.arange(2, dtype=torch.int32, device="cuda"))
+
+
+def step(kt, descriptors, inputs=None):
+    tokens, off, idx, slots = inputs or step_inputs()
+    return kt.derive_lookup_store(tokens, off, idx, descriptors, slots)
 
 
 @pytest.mark.parametrize("side_stream", [False, True])
 @pytest.mark.parametrize("extra", [False, True])
 def test_calls_in_flight_keep_their_encodings(side_stream, extra):
+    """60 calls enqueued behind 0.3 s of work on the table's stream.  (With appended dimensions some calls take the copies
+    from pageable memory, which wait for the current stream.)"""
     rng = np.random.default_rng(3)
-    torch.cuda.synchronize()
     stream = torch.cuda.Stream() if side_stream else None
     kt = KeyTable(4, 8, stream=stream)
+    inputs = step_inputs()
     batches = [[desc(rng, 10 * k + j, extra) for j in range(1 + k % 7)] for k in range(60)]
-    got = []
-    for b in batches:
-        with torch.cuda.stream(stream):
-            torch.empty(1 << 22, device="cuda").fill_(1.0)  # keeps the stream busy behind the host
-        got.append(step(kt, b)[0])
+    for b in batches[:7]:
+        step(kt, b, inputs)
+    # (a pinned allocation that the cache cannot serve waits for the device)
+    pinned = [torch.empty(1 << k, dtype=torch.uint8, pin_memory=True) for k in range(7, 14) for _ in batches]
+    del pinned
+    a = torch.ones((4096, 4096), device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for _ in range(150):
+            a = a @ a * 0.0 + 1.0
+        done = torch.cuda.Event()
+        done.record()
+    got = [step(kt, b, inputs) for b in batches]
+    assert extra or not done.query()
     torch.cuda.synchronize()
     kt.check()
-    for b, d in zip(batches, got):
-        assert np.array_equal(d.cpu().numpy(), O.descriptor_digests(b))
+    for b, out in zip(batches, got):
+        assert np.array_equal(out[0].cpu().numpy(), O.descriptor_digests(b))
     kt.close()
 
 
