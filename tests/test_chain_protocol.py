@@ -1,8 +1,9 @@
-"""CPU model of the chain kernel's two-warp protocol (csrc/pk_derive.cu, k_chain).
+"""CPU model of the two-warp protocols of a pair: the chains (csrc/pk_derive.cu, k_chain and k_chain_split) and the
+digests of few messages (csrc/pk_pair.cuh, pair_schedule and pair_rounds).
 
-Each layout's rounds warp (R) and schedule warp (S) are written out as their
+Each protocol's rounds warp (R) and schedule warp (S) are written out as their
 sequences of named-barrier operations and shared-memory accesses, step by step
-as the kernel issues them; every interleaving of the two warps is explored and
+as the kernels issue them; every interleaving of the two warps is explored and
 must end with both warps done (no deadlock), no warp arriving twice in one
 phase of a barrier (count 64: one arrival per warp completes a phase), no
 pending arrival left at the end, and no read of a buffer overlapping the other
@@ -13,31 +14,9 @@ import pytest
 # ops: ("arrive", id) | ("sync", id) | ("w+", buf) | ("w-", buf) | ("r+", buf) | ("r-", buf)
 
 
-def one_pair(n):
-    """One pair per CTA: barriers 1-3 block-1 slices, 4 block 2 ready, 5 k published."""
-    S = [("w+", "kw2_0"), ("w-", "kw2_0"), ("arrive", 4)]
-    for i in range(n):
-        if i > 0:
-            S += [("sync", 5), ("r+", "kpub"), ("r-", "kpub"), ("arrive", 4)]
-        slices = 6 if i + 1 < n else 3
-        for sl in range(1, slices + 1):
-            buf = f"kw1_{sl}" if sl <= 3 else f"kw2_{(i + 1) & 1}"
-            S += [("w+", buf), ("w-", buf)]
-            if sl <= 3:
-                S += [("arrive", sl)]
-    R = []
-    for i in range(n):
-        for sl in (1, 2, 3):
-            R += [("sync", sl), ("r+", f"kw1_{sl}"), ("r-", f"kw1_{sl}")]
-        R += [("sync", 4), ("r+", f"kw2_{i & 1}"), ("r-", f"kw2_{i & 1}")]
-        if i + 1 < n:
-            R += [("w+", "kpub"), ("w-", "kpub"), ("arrive", 5)]
-    return R, S
-
-
-def four_pairs(n):
-    """Four pairs per CTA, one pair's barriers: s1 (block-1 slice 1, and block 2 of the step ready), s1b
-    (block-1 slices 2-3), k (k published)."""
+def chain(n):
+    """n steps of a pair of either chain: barriers s1 (block-1 slice 1, and block 2 of the step ready), s1b (block-1
+    slices 2-3), k (k published)."""
     S = [("w+", "kw2_0"), ("w-", "kw2_0")]
     for i in range(n):
         if i > 0:
@@ -54,6 +33,34 @@ def four_pairs(n):
         if i + 1 < n:
             R += [("w+", "kpub"), ("w-", "kpub"), ("arrive", "k")]
     return R, S
+
+
+def ring(n, pad=False):
+    """n blocks of a pair's messages through the two-stage ring: barriers filled_0/1 and read_0/1; `pad`: then the
+    constant last block, from no ring.  The rounds warp reads the next block's first words before it marks a stage read."""
+    S = []
+    for b in range(n):
+        if b >= 2:
+            S += [("sync", f"read_{b & 1}")]
+        S += [("w+", f"kw_{b & 1}"), ("w-", f"kw_{b & 1}"), ("arrive", f"filled_{b & 1}")]
+
+    def first_words(b):
+        return [("sync", f"filled_{b & 1}"), ("r+", f"kw_{b & 1}"), ("r-", f"kw_{b & 1}")] if b < n else []
+
+    total = n + pad
+    R = first_words(0)
+    for b in range(total):
+        if b < n:
+            R += [("r+", f"kw_{b & 1}"), ("r-", f"kw_{b & 1}")]
+        if b + 1 < total:
+            R += first_words(b + 1)
+        if b + 2 < n:
+            R += [("arrive", f"read_{b & 1}")]
+    return R, S
+
+
+def ring_and_pad(n):
+    return ring(n, True)
 
 
 class ProtocolError(Exception):
@@ -134,7 +141,7 @@ def explore(R, S):
     return len(seen), finals
 
 
-@pytest.mark.parametrize("layout", [one_pair, four_pairs])
+@pytest.mark.parametrize("layout", [chain, ring, ring_and_pad])
 @pytest.mark.parametrize("n", [1, 2, 3, 5])
 def test_protocol_has_no_deadlock_double_arrival_or_race(layout, n):
     states, finals = explore(*layout(n))
@@ -152,25 +159,36 @@ def _mutate(prog, i, new=None):
 
 def test_model_catches_a_missing_sync():
     """Without the rounds warp's wait for block-1 slice 2, its read can overlap the schedule warp's write."""
-    R, S = four_pairs(3)
+    R, S = chain(3)
     i = R.index(("sync", "s1b"))
     with pytest.raises(ProtocolError):
         explore(_mutate(R, i), S)
 
 
 def test_model_catches_a_double_arrival():
-    """The schedule warp marking block 2 ready on its own barrier again before the rounds warp has synced
-    the previous phase: a second arrival in one phase."""
-    R, S = one_pair(3)
-    j = S.index(("sync", 5))
+    """The schedule warp marking the first slice of the next step without waiting for k: a second arrival in one phase
+    of its barrier, or a read of k under its write."""
+    R, S = chain(3)
+    j = S.index(("sync", "k"))
     with pytest.raises(ProtocolError):
         explore(R, _mutate(S, j))
+
+
+def test_model_catches_a_ring_stage_filled_too_early():
+    """The schedule warp not waiting until a stage is read; the rounds warp marking it read before its last words."""
+    R, S = ring(5)
+    with pytest.raises(ProtocolError):
+        explore(R, _mutate(S, S.index(("sync", "read_0"))))
+    i = R.index(("arrive", "read_0"))
+    early = R[:1] + [R[i]] + R[1:i] + R[i + 1:]
+    with pytest.raises(ProtocolError):
+        explore(early, S)
 
 
 def test_model_catches_a_buffer_reused_too_early():
     """Block 2 single-buffered (always kw2_0): the schedule warp would overwrite the buffer the rounds warp
     is still reading."""
-    R, S = four_pairs(3)
+    R, S = chain(3)
     S = [(op, "kw2_0" if isinstance(a, str) and a.startswith("kw2_") else a) for op, a in S]
     R = [(op, "kw2_0" if isinstance(a, str) and a.startswith("kw2_") else a) for op, a in R]
     with pytest.raises(ProtocolError):
@@ -179,7 +197,7 @@ def test_model_catches_a_buffer_reused_too_early():
 
 def test_model_catches_a_deadlock():
     """The schedule warp waiting for k before it has marked the step's first slice (i = 0 included)."""
-    R, S = four_pairs(2)
+    R, S = chain(2)
     S = [("sync", "k")] + S
     with pytest.raises(ProtocolError):
         explore(R, S)
