@@ -407,8 +407,8 @@ int pk_key_strings(const uint8_t *keys_dev, uint64_t n, const char *prefix, uint
  *                     once. */
 /* Test hook of pk_evict's bounded grid barriers (no paper counterpart): the
  * same launch as pk_evict(ctx, budget, budget, ...) with the barrier waits
- * bounded at spin_limit polls of about 100-200 ns (> 0; at most the default
- * of about a second) and CTA 0 withholding its arrival at the first barrier,
+ * bounded at spin_limit polls of about 230 ns (> 0; at most the default
+ * of about 2 s) and CTA 0 withholding its arrival at the first barrier,
  * so that every other CTA's wait runs out.  Needs stamps attached and more
  * than `budget` entries in the table (else the kernel returns before the
  * barrier) and a table of at least 2^10 entries (two CTAs or more).  The

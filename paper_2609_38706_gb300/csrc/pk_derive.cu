@@ -665,8 +665,8 @@ __device__ __forceinline__ void schedule16(uint32_t w[16], uint4 (*out)[kChainLa
 
 // rounds t = 16q .. 16q+15 with K+W from shared memory
 // (the 16 words are read into registers before the first round: a lone warp
-// runs 64 rounds in 2018 instead of 2241 cycles when no round waits on its
-// shared-memory read)
+// runs 64 rounds in 1917 instead of 2184 cycles, in the late form 1830 instead
+// of 2233, when no round waits on its shared-memory read)
 template <int F>
 __device__ __forceinline__ void rounds16_kw(uint32_t v[8], const uint4 (*kw)[kChainLanes], int q, uint32_t lane,
                                             uint32_t one) {
@@ -919,7 +919,7 @@ k_chain(const int64_t *key_off, const uint32_t *desc_idx,
 // as a loop of 16 rounds: long-context key derivation 938 -> 1013 us), each
 // 16 words of K + W read while the 16 rounds before them run, and each barrier synced
 // some slots before the words it guards are needed.  The schedule warp's work
-// still costs the rounds warp about 8% (857 us with its arithmetic removed):
+// still costs the rounds warp about 5% (865 -> 824 us with its arithmetic removed):
 // its shared-memory traffic is kept to 16-byte vectors (938 -> 924 us) and its
 // slices run one copy of the code.  Long-context key derivation (64 chains of
 // 512 steps) 1060 -> 925 us against one lane per request, 865 us with the
@@ -1187,7 +1187,8 @@ unsigned grid_for(uint64_t n, unsigned block) { return (unsigned)((n + block - 1
 
 // Dynamic shared memory of the kernels whose CTAs must not stack on an SM: padded past half of an SM's, or past a
 // third for two per SM (a launch that becomes resident while its predecessor drains otherwise stacks CTAs on the SMs
-// that free up first).
+// that free up first).  The price: while such a CTA runs, a CTA of another stream's kernel comes up on its SM only if
+// it needs no more shared memory than is left (227 KB less 116, or less one or two times 76).
 constexpr size_t kOnePerSm = 116 * 1024;
 constexpr size_t kTwoPerSm = 76 * 1024;
 static_assert(kOnePerSm >= kChainPairs * sizeof(ChainSmem) && kOnePerSm >= 4 * sizeof(SplitSmem) &&
@@ -1265,9 +1266,11 @@ cudaError_t pk_launch_derive_enc(const pk_ctx *ctx, const int32_t *tokens, uint6
                           (const int64_t *)key_off, 0u, C, pad, keys, dw, one);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
-    // The multiply-add round form pays once two warps of chunks share an SM sub-partition (two warps 4766 against
-    // 5191 cycles per compression each, a lone one 3170 against 2830; long-context key derivation, 1.7 warps per
-    // sub-partition, 870.7 -> 868.1 us).  With an unknown SM count the compiler's form is kept.
+    // The multiply-add round form from more than one warp of chunks per SM sub-partition (two warps 4610 against 5334
+    // cycles per compression each; long-context key derivation, 1.7 warps per sub-partition, 870.7 -> 868.1 us).  Below
+    // the line the two forms are close: key derivation at half a warp per sub-partition, compiler's form | multiply-add,
+    // in us: chunks of 16 23.6 | 23.8, of 64 28.1 | 28.0, of 256 57.8 | 56.6; at one warp 26.3 | 25.9, 35.2 | 33.8,
+    // 78.7 | 73.3.  With an unknown SM count the compiler's form is kept.
     const uint64_t warps = (most + 31) / 32;
     const bool fma = ctx->sm_count > 0 && warps > 4ull * ctx->sm_count;
     const unsigned grid = grid_for(most, kDigestBlock) + dw.desc_blocks;

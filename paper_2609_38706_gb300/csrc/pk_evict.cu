@@ -55,7 +55,7 @@ constexpr uint32_t kEvThreads = 512;
 constexpr uint32_t kEvBlocks = 2;  // CTAs per SM
 constexpr uint32_t kEvRows = 512;  // table entries per CTA below which no further CTA is launched
 constexpr uint32_t kPasses = 7;    // histogram rows of the passes within a call, used in turn
-constexpr uint32_t kSpinLimit = 1u << 23;  // x ~100 ns: a barrier gives up after about a second
+constexpr uint32_t kSpinLimit = 1u << 23;  // polls of about 230 ns: a barrier gives up after about 2 s
 
 struct EvictHeader {  // zeroed by the host before every launch
     unsigned int arrive;             // CTAs that have arrived at the grid barriers so far

@@ -76,7 +76,7 @@ cudaError_t pk_launch_compare_pages(const uint32_t *slots, const uint8_t *pages,
                                     int32_t *status, cudaStream_t s);
 uint64_t pk_evict_scratch_bytes_impl(uint64_t capacity);
 // spin_limit: polls of a barrier wait before it gives up (0 = the default of
-// about a second); withhold_first_cta: CTA 0 does not arrive at the first
+// about 2 s); withhold_first_cta: CTA 0 does not arrive at the first
 // barrier (the timeout test).
 cudaError_t pk_launch_evict(const pk_ctx *ctx, uint64_t budget, uint64_t keep, void *scratch, uint32_t *evicted,
                             uint64_t evicted_cap, unsigned long long *n_evicted, int32_t *status, cudaStream_t s,

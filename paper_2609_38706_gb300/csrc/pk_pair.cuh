@@ -9,7 +9,9 @@
 //
 // With few messages the SM sub-partitions have room and a message's serial
 // blocks set the time: one lane per message, schedule in the same thread,
-// takes 2460 cycles per 64-byte block (a lone warp, measured), a pair 1600.
+// takes a lone warp 2719 to 2926 cycles per 64-byte block by the form of its
+// additions, a pair alone on its SM 1793, each of two pairs 2204, of three 2414
+// (their schedule warps share a sub-partition).
 // A CTA holds up to three pairs, their rounds warps (0, 1, 2) on a
 // sub-partition each and their schedule warps (3, 7, 11) on the fourth; warps
 // 4-6 and 8-10 do nothing.  Beyond 48 messages per SM the pairs would share
@@ -79,7 +81,9 @@ __device__ __forceinline__ void pair_tables(PairSmem &sm, const uint32_t *pad_kw
     for (uint32_t t = threadIdx.x; t < kPairRow; t += kPairThreads) sm.zero[t] = 0u;
 }
 
-// Named barriers of pair p: 1 + 4p, 2 + 4p a ring stage filled, 3 + 4p, 4 + 4p a stage read.
+// Named barriers of pair p: 1 + 4p, 2 + 4p a ring stage filled, 3 + 4p, 4 + 4p a stage read.  Of the kernels that use
+// the pairs, the warps without a part release the successor at once, which becomes resident as far as the pairs leave
+// room and waits there.
 //
 // Schedule warp: K+W of `blocks` blocks.  src.load(b, t) is word t (0..15) of
 // block b of this lane's message in memory (0 past its last whole word;

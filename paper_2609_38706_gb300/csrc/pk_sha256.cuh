@@ -213,12 +213,15 @@ namespace pk {
 // rate and alongside the ALU (an SHF/IMAD pair: 2.1 cycles).  The two round
 // forms differ only in where the additions go, never in the value computed:
 //   kAddsPlain  the compiler's choice (ALU-bound at 25 cycles per round when
-//               the sub-partition is saturated, 29.8 for a lone warp);
+//               the sub-partition is saturated, 30 for a lone warp);
 //   kAddsFma    every addition as x * one + y on the FMA pipe (`one` is a
-//               run-time 1 the compiler cannot fold): 22.2 cycles per round
-//               and 10-13% faster compressions once 4 or more warps share a
-//               sub-partition, but 33.4 cycles for a lone warp (the
-//               multiply-add's longer latency sits on the critical path);
+//               run-time 1 the compiler cannot fold): 22 cycles per round when
+//               saturated, 33 for a lone warp's rounds alone (the
+//               multiply-add's longer latency sits on their critical path);
+//               with the schedule beside them (compress_rolled, in a loop of
+//               its own) a compression takes each of 1, 2 and 4 warps on a
+//               sub-partition 2719, 4610 and 8926 cycles against 2926, 5334
+//               and 10563 in the plain form;
 //   kAddsLate   (rounds only) one 3-input add after each set of rotations,
 //               e' = S1 + Ch + (d + h + kw) and a' = e' + S0 + (Maj - d), the
 //               sums in brackets made beside them, two of them on the FMA pipe:
@@ -331,10 +334,10 @@ __device__ __forceinline__ void compress_kw(uint32_t st[8], const uint32_t *__re
 // the half-rate ALU, a 3-input xor, a 3-input add: 20.7 cycles, measured), not
 // by throughput; one lane per message runs two such chains and all their
 // operations through the one pipe (10 logic operations and the adds).  Measured
-// on GB300, cycles per 64 rounds of a lone warp with K + W in shared memory: 2637
-// with one lane per message (round_kw), 1488 with two; with two warps per SM
-// sub-partition 2520 for 2 x 16 messages, so a full sub-partition is better
-// served by one lane per message.
+// on GB300, cycles per 64 rounds of a lone warp with K + W in shared memory, 16
+// words read ahead: 1917 with one lane per message (round_kw), 1484 with two; of
+// each of two warps on a sub-partition 3256 and 2483, the first for twice the
+// messages, so a full sub-partition is better served by one lane per message.
 // The select is written over P and Q, made a slot ahead of their use:
 // Ch = e ? f : g, Maj = a ? (b | c) : (b & c).
 // ---------------------------------------------------------------------------
@@ -359,7 +362,7 @@ struct SplitState {
 };
 
 // The select's operands for a slot with x1 = b and x2 = c: Q = c or b & c, and P = b or b | c as (b + c) - Q on
-// the FMA pipe (a lone warp's 64 rounds 1598 cycles with P as a logic operation, 1488 so).
+// the FMA pipe (a lone warp's 64 rounds 1598 cycles with P as a logic operation, 1484 so).
 __device__ __forceinline__ void split_select(SplitState &v, const SplitLane &l, uint32_t b, uint32_t c) {
     v.Q = c & (b | ~l.maj);
     v.P = mad1(v.Q, l.minus, mad1(c, l.one, b));
